@@ -62,6 +62,7 @@ void free_patch(igafd_patch *P) {
   cudaFree(P->eig_work); cudaFree(P->eig_jobs); cudaFree(P->coef);
   cudaFree(P->lfeat); cudaFree(P->lybar);
   igafd_fd_tc_free(P);
+  igafd_fd_split_free(P);
   igafd_adi_free(P);
   for (int i = 0; i < IGAFD_NEV; ++i)
     if (P->ev[i]) cudaEventDestroy(P->ev[i]);
@@ -153,6 +154,7 @@ igafd_status build(igafd_patch *P, const igafd_patch_desc *d, cudaStream_t s) {
 igafd_status igafd_build_prec(igafd_patch *P, cudaStream_t s) {
   IGAFD_TRY(igafd_setup_pencils_eig(P, s, P->scaled ? P->wK : nullptr, P->scaled ? P->wM : nullptr));
   IGAFD_TRY(igafd_fd_tc_init(P, s));   // also the FP32 copies U32_k
+  IGAFD_TRY(igafd_fd_split_init(P, s));
   IGAFD_CUDA(cudaStreamSynchronize(s));
   return IGAFD_OK;
 }

@@ -71,7 +71,8 @@ enum {
   S_COUNT
 };
 
-struct FDMixed;   // mixed-precision FD workspace (fd_mixed.cu)
+struct FDMixed;   // mixed-precision FD workspace (fd_tc.cu)
+struct FDSplit;   // digit images of the FP64 FD on the tensor cores (fd_split.cu)
 
 struct igafd_patch {
   int dev;
@@ -85,7 +86,9 @@ struct igafd_patch {
   int twin[3];                  // smallest direction with the same knot vector (same 1D pencils)
   double *ctrl;                 // [dim][gm_d]..[gm_1]
   double *kctrl;                // coefficient control values [km_d]..[km_1] or null
-  // generalized eigenpairs: U[k][i*n + j], D[k][j]; inv_lam[N] = 1/(D1+D2+D3)
+  // generalized eigenpairs: U[k][i*n + j], D[k][j]; inv_lam[N] = 1/(D1+D2+D3), indexed like a
+  // dof vector, or [j_1][j_3][j_2] where the FP64 FD runs on the tensor cores (fd_split.cu);
+  // inv_lam32 always indexed like a dof vector
   double *U[3], *D[3];
   float *U32[3];
   double *inv_lam;
@@ -125,6 +128,7 @@ struct igafd_patch {
   double *coef;                 // [2 * IGAFD_COEF_CAP]: alpha_k, beta_k of the last solve
   double *host_scal;            // pinned mirror of scal
   FDMixed *mixed;
+  FDSplit *split;               // null: n_k > 128 in some direction
   double *wK[3], *wM[3];        // span scalings of the pencils (device, null = unscaled)
   int fd_fused;                 // 1: fused tensor-core FD (3 kernels) when n_k <= 128
   int fd_fused_op[3];           // the same per operand type (TF32, BF16, FP16), set by the autotuner
@@ -172,6 +176,12 @@ igafd_status igafd_adi_apply(igafd_patch *P, const double *r, double *z, cudaStr
 // FD apply; kernels do nothing while *done_flag != 0 (done_flag may be null)
 igafd_status igafd_fd64_apply(igafd_patch *P, const double *r, double *z, cudaStream_t s,
                               double *done_flag);
+// FP64 FD on the tensor cores (every n_k <= 128)
+bool igafd_fd_split_shape(const igafd_patch *P);
+igafd_status igafd_fd_split_init(igafd_patch *P, cudaStream_t s);
+void igafd_fd_split_free(igafd_patch *P);
+igafd_status igafd_fd_split_apply(igafd_patch *P, const double *r, double *z, cudaStream_t s,
+                                  double *done_flag);
 igafd_status igafd_fd32_apply(igafd_patch *P, const double *r, double *z, cudaStream_t s,
                               double *done_flag);
 igafd_status igafd_fd_tc_apply(igafd_patch *P, igafd_dtype dt, const double *r, double *z,

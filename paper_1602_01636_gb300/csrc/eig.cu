@@ -1090,6 +1090,29 @@ __global__ void inv_lambda_kernel(const double *D1, const double *D2, const doub
   inv32[i] = (float)r;
 }
 
+// The same values, inv in the layout [i_1][i_3][i_2] of the tensor-core FP64
+// FD: blocks of 32 x 32 (i_1, i_2) at one i_3, transposed in shared memory.
+__global__ void __launch_bounds__(256) inv_lambda_t_kernel(const double *D1, const double *D2,
+                                                           const double *D3, int n1, int n2, int n3,
+                                                           double *inv, float *inv32) {
+  __shared__ double t[32][33];
+  const int a0 = blockIdx.x * 32, b0 = blockIdx.y * 32, i3 = blockIdx.z;
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const double d3 = D3 ? D3[i3] : 0.0;
+  for (int b = w; b < 32; b += 8) {
+    const int i1 = a0 + l, i2 = b0 + b;
+    if (i1 >= n1 || i2 >= n2) continue;
+    const double r = 1.0 / (D1[i1] + D2[i2] + d3);
+    t[b][l] = r;
+    inv32[((long long)i3 * n2 + i2) * n1 + i1] = (float)r;
+  }
+  __syncthreads();
+  for (int a = w; a < 32; a += 8) {
+    const int i1 = a0 + a, i2 = b0 + l;
+    if (i1 < n1 && i2 < n2) inv[((long long)i1 * n3 + i3) * n2 + i2] = t[l][a];
+  }
+}
+
 }  // namespace
 
 static GemmJob gemm_job(int n, int transA, const double *A, const double *B, const double *D,
@@ -1253,9 +1276,14 @@ igafd_status igafd_setup_pencils_eig(igafd_patch *P, cudaStream_t s, const doubl
     IGAFD_CUDA(cudaMemcpyAsync(P->D[k], P->D[k0], n * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
   long long N = P->N;
-  inv_lambda_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(
-      P->D[0], P->D[1], dim == 3 ? P->D[2] : nullptr, P->n[0], P->n[1], N, P->inv_lam,
-      P->inv_lam32);
+  if (igafd_fd_split_shape(P))
+    inv_lambda_t_kernel<<<dim3((P->n[0] + 31) / 32, (P->n[1] + 31) / 32, P->n[2]), 256, 0, s>>>(
+        P->D[0], P->D[1], dim == 3 ? P->D[2] : nullptr, P->n[0], P->n[1], P->n[2], P->inv_lam,
+        P->inv_lam32);
+  else
+    inv_lambda_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(
+        P->D[0], P->D[1], dim == 3 ? P->D[2] : nullptr, P->n[0], P->n[1], N, P->inv_lam,
+        P->inv_lam32);
   IGAFD_LAUNCHED(1);
   IGAFD_CUDA(cudaGetLastError());
   // route taken per pencil (0 fast, 1 FP64 Jacobi, 2 failed) and the error flag

@@ -163,6 +163,7 @@ GemmArgs mode_args(const int *n, int dim, int k, const void *U, bool forward, co
 // FP64: every product and the divide in FP64 (FD == P^{-1} up to rounding).
 igafd_status igafd_fd64_apply(igafd_patch *P, const double *r, double *z, cudaStream_t s,
                               double *done_flag) {
+  if (P->split) return igafd_fd_split_apply(P, r, z, s, done_flag);
   const int dim = P->dim;
   const double *in = r;
   double *bufs[2] = {P->fd_a, P->fd_b};

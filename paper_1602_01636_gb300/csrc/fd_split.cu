@@ -1,0 +1,685 @@
+// FP64 fast-diagonalization apply on the tensor cores, for n_k <= 128.
+//
+// GB300 issues two FP64 FMAs per clock per SM (1.26 TFLOP/s in all), so the
+// 12 n^4 FLOP of the six mode products take 2.6 ms at n = 128 on the FP64
+// pipe however they are arranged (the SIMT kernel of fd.cu measured 3.10 ms).
+// Here each FP64 operand is split into six 10-bit integer digits (the
+// splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012, with
+// integer digits), and the products of digits run on the tensor cores:
+//
+//   a_mi = 2^(ea_m - 1081) sum_s da[s]_mi 1024^(5 - s),   |da[s]| <= 512
+//   b_ji = 2^(eb_j - 1082) sum_t db[t]_ji 1024^(5 - t),   |db[t]| <= 512
+//   sum_i a_mi b_ji = 2^(ea_m + eb_j - 2163) sum_g 1024^(10 - g) G_g,
+//   G_g = sum_{s + t = g} sum_i da[s]_mi db[t]_ji
+//
+// with ea_m the largest exponent field of row m and eb_j that of row j of B
+// (U_k^T or U_k, split at set-up). Digits are exact in FP16; the FP32
+// accumulators of tcgen05.mma hold the leading groups' integers exactly (see
+// kStepTab). Groups g <= 5 are kept (21 digit products); their accumulators
+// are summed as 64-bit integers and rounded to FP64 once. In units of 2^-53
+// of the result's norm, a product's error is 0.4-1.8 (0.4 unless one factor's
+// entries decay along the sum) where the FP64 FMA chain of the SIMT kernel
+// has 1.0 (K = 12) to 4.8 (K = 128). The divide by D_1 (+) D_2 (+) D_3
+// multiplies the integer result before that rounding. No FP64 instruction is
+// executed (each would issue at the 2-per-clock rate).
+//
+// Measured: 181 us per apply at n = 128 (SIMT: 3.10 ms), 103 us at
+// (95, 61, 77) (SIMT: 0.98 ms). A pass at n = 128 (about 25 us) is bound by
+// integer instructions (64 lanes per clock per SM): splitting the rows 4 us,
+// the MMAs with the summation of their accumulators 9 us (the MMAs alone 5),
+// rounding 5 us, the rest loads and the launch.
+//
+// A CTA takes 128 rows (the other directions' indices) and up to 128 columns.
+// A's digits live in tensor memory (6 slices of K/2 columns: 384 of 512 at
+// K = 128), where each thread writes the digits of its own row; B's digits
+// lie in shared memory (6 x 32 KB at n = 128); two accumulators of kNS columns
+// take the rest of tensor memory: one warp issues the products of a step into
+// one while the other warps read the previous one.
+//
+// Directions are contracted in the order 3, 2, 1 and back 1, 3, 2: in four of
+// the six products (three of four in 2D) the row index is then contiguous in
+// memory and rows map to lanes without a transposition; the other two read
+// rows that are contiguous in the contracted direction through a
+// warp-private transposition. The divide's table inv_lam is stored in the
+// layout the third product writes, [j1][j3][j2].
+#include "common.cuh"
+
+#include <atomic>
+#include <cstdlib>
+#include <type_traits>
+
+#include <cuda_fp16.h>
+
+namespace {
+
+constexpr int kM = 128;                 // rows per CTA (MMA M, TMEM lanes)
+constexpr int kWorkers = 512;           // 4 warps per lane quarter; one more warp issues copies and MMAs
+constexpr int kThreads = kWorkers + 32;
+constexpr int kSlices = 6;              // digits per operand
+constexpr int kBits = 10;               // bits per digit
+constexpr int kNS = 64;                 // columns per accumulator
+constexpr int kFirst = 3;               // slices of B fetched before the input is read
+constexpr int kTrans = 16 * 32 * 17 * 8;// bytes of the transposition buffers
+constexpr long long kSpin = 1ll << 26;  // bounded waits
+// X + kBias = sum_s (digit_s + 512) 1024^(5-s): every 10-bit field is then the
+// digit plus 512
+constexpr unsigned long long kBias = 512ull * (1ull + (1ull << 10) + (1ull << 20) + (1ull << 30) +
+                                               (1ull << 40) + (1ull << 50));
+
+struct SplitArgs {
+  const double *in;
+  double *out;
+  long long M;            // rows
+  int F;                  // rows m = hi F + lo
+  long long in_hi, in_lo, in_k, out_hi, out_lo, out_n;   // element strides
+  int K, Kp;              // contracted length, padded to a multiple of 32
+  int N, Np, NT;          // columns, padded to 16; columns per CTA (multiple of 16)
+  const unsigned char *img;   // digits of B: [slice][64-wide K chunk][Np][128 B], swizzled
+  const int *eb;              // exponent field of each row of B
+  const double *inv_lam;      // divide table, indexed like out (null: none)
+  const double *done;
+  int *err;
+};
+
+// The accumulation steps of a column block for K <= 64 and K <= 128: the
+// group, and its 64-wide K chunks c0 <= c < c1. FP32 accumulation of integers
+// is exact below 2^24, and the chunks keep the sums of the leading groups
+// there: |a_0 b_0| <= 2^17 over 128 terms; the products of groups 1 and 2 have
+// |a| <= 2^9 and, over U_k's entries, |b| of half its 2^9 on average, so their
+// sums over 64 terms stay below 2^23 per product (2^22 with a_0). Group 3
+// weighs 2^-30 of group 0: a rounding there is below the result's last bit.
+struct Step { signed char g, c0, c1; };
+__constant__ Step kStepTab[2][8] = {
+    {{0, 0, 2}, {1, 0, 2}, {2, 0, 2}, {3, 0, 2}, {4, 0, 2}, {5, 0, 2}},
+    {{0, 0, 2}, {1, 0, 1}, {1, 1, 2}, {2, 0, 1}, {2, 1, 2}, {3, 0, 2}, {4, 0, 2}, {5, 0, 2}}};
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
+// K-major, 128-byte swizzle (8-row groups of 1024 B)
+__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)(16 >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
+// Bounded wait, given up early once another thread's wait ran out.
+__device__ __forceinline__ bool wait_on(uint64_t *bar, uint32_t parity, const int *failed) {
+  for (long long it = 0; it < kSpin; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if ((it & 255) == 255 && *(volatile const int *)failed) return false;
+  }
+  return false;
+}
+__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// shifts by 32 or more give 0
+__device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t s) {
+  uint32_t r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
+  return r;
+}
+
+// The exponent field of a double given its high word: 1 for zero and
+// subnormals (whose mantissa has no hidden bit), 0x7ff for infinities and NaN.
+__device__ __forceinline__ int exp_field(uint32_t hi) {
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  return e > 1 ? e : 1;
+}
+
+// X + kBias with X = d 2^(1023 + BITS - ea) truncated, |X| < 2^BITS, as its
+// upper and lower 30 bits (junk above bit 30 of the lower word). A has 58
+// bits, so that its top digit fits the packed conversion; B has 59.
+template <int BITS>
+__device__ __forceinline__ void biased_fixed(double d, int ea, uint32_t &w1, uint32_t &w0) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  // mantissa with the hidden bit at bit 63 (its place holds the exponent's
+  // lowest bit, which is 0 where there is no hidden bit)
+  const uint32_t mh = __funnelshift_l(lo, hi, 11) | ((hi & 0x7ff00000u) ? 0x80000000u : 0u);
+  const uint32_t ml = lo << 11;
+  const uint32_t sh = (uint32_t)(ea + 64 - BITS - exp_field(hi));
+  const uint32_t s1 = min(sh, 32u);
+  uint32_t xh = shr_clamp(mh, s1);
+  uint32_t xl = shr_clamp(__funnelshift_rc(ml, mh, s1), sh - s1);
+  const uint32_t sg = (uint32_t)((int)hi >> 31);
+  const unsigned long long x =
+      (((unsigned long long)(xh ^ sg) << 32) | (xl ^ sg)) + kBias;
+  w0 = (uint32_t)x;
+  w1 = __funnelshift_r(w0, (uint32_t)(x >> 32), 30);
+}
+
+// digit at bit 10 POS of the words of two elements, as packed FP16 (element 0
+// in the low half): fields 0..1023 become 1024 + field by their bits, minus 1536
+template <int POS> __device__ __forceinline__ uint32_t digit2(uint32_t a, uint32_t b) {
+  uint32_t w;
+  if (POS == 0) w = __byte_perm(a, b, 0x5410);
+  else if (POS == 1) w = __byte_perm(a, b, 0x6521) >> 2;
+  else w = __byte_perm(a, b, 0x7632) >> 4;
+  w = (w & 0x03ff03ffu) | 0x64006400u;
+  const __half2 h = __hsub2(*reinterpret_cast<__half2 *>(&w), __half2half2(__ushort_as_half(0x6600)));
+  return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// T 2^E lam for what round_fixed leaves out (noinline: rare)
+__device__ __noinline__ double round_slow(long long T, int E, double lam) {
+  return ldexp((double)T, E) * lam;
+}
+
+// T 2^E (times lam with LAM) rounded to FP64 with integer instructions; slow
+// is set, and the value undefined, for results outside the normal range and
+// for lam that is not a positive normal number
+template <bool LAM>
+__device__ __forceinline__ double round_fixed(long long T, int E, double lam, bool &slow) {
+  const int sg = (int)(T >> 63);
+  const unsigned long long u = (unsigned long long)(T ^ (long long)sg) - (unsigned long long)(long long)sg;
+  uint32_t h = (uint32_t)(u >> 32), l = (uint32_t)u;
+  int e = E + 1085 + 1;                             // exponent field of the result minus 1, and 1
+  if (h == 0u) { h = l; l = 0u; e -= 32; }
+  const int lz = __clz((int)h);
+  h = __funnelshift_l(l, h, lz);
+  l = l << (lz & 31);
+  e -= lz;                                          // (h l) in [2^63, 2^64), or 0
+  if (LAM) {
+    const uint32_t lh = (uint32_t)__double2hiint(lam), ll = (uint32_t)__double2loint(lam);
+    slow = slow || lh - 0x00100000u >= 0x7fe00000u;
+    // the upper half of the 128-bit product, but for the carry of its lower half (2^-63)
+    const uint32_t Lh = __funnelshift_l(ll, lh, 11) | 0x80000000u, Ll = ll << 11;
+    const unsigned long long p = (unsigned long long)h * Lh + __umulhi(h, Ll) + __umulhi(l, Lh);
+    h = (uint32_t)(p >> 32);
+    l = (uint32_t)p;
+    const int n = (int)(~h >> 31);                  // one more shift
+    h = __funnelshift_l(l, h, n);
+    l <<= n;
+    e += (int)(lh >> 20) - 1022 - n;
+  }
+  // 53 bits and the rounding bit; a carry runs into the exponent field
+  const unsigned long long q =
+      (((unsigned long long)(h >> 11) << 32) | __funnelshift_r(l, h, 11)) + ((l >> 10) & 1u) +
+      ((unsigned long long)(uint32_t)(e - 1) << 52);
+  const bool zero = T == 0;
+  slow = slow || (!zero && (uint32_t)(e - 2) >= 2043u);
+  return __hiloint2double(zero ? 0 : (int)((uint32_t)(q >> 32) | ((uint32_t)sg & 0x80000000u)),
+                          zero ? 0 : (int)(uint32_t)q);
+}
+
+template <bool LAM>
+__global__ void __launch_bounds__(kThreads, 1) split_pass_kernel(SplitArgs a) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *sB = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  __shared__ uint64_t bar_b[2], bar_a[kSlices], bar_full[2], bar_empty[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ unsigned short s_ea[4][kM], s_eb[kM];
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n0 = (int)blockIdx.y * a.NT;
+  const int NTc = a.Np - n0 < a.NT ? a.Np - n0 : a.NT;     // columns of this CTA
+  const int nkc = (a.Kp + 63) >> 6;
+  const int slice_bytes = nkc * a.NT * 128;
+  const int scols = a.Kp >> 1;                             // TMEM columns per slice of A
+  const int dbase = kSlices * scols;                       // accumulators: 2 x kNS columns
+  const int two = nkc > 1 ? 1 : 0;
+  const int per = two ? 8 : 6;                             // steps per column block
+  const int nsub = (NTc + kNS - 1) / kNS;
+  const bool issuer = tid == kWorkers;                     // lane 0 of the last warp
+
+  if (issuer) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bar_b[i], 1);
+      mbar_init(&bar_full[i], 1);
+      mbar_init(&bar_empty[i], kWorkers / 32);
+    }
+    for (int i = 0; i < kSlices; ++i) mbar_init(&bar_a[i], kWorkers / 32);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_fail = 0;
+  }
+  auto load_slices = [&](int s0, int s1, uint64_t *bar) {   // one thread
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+                 "r"((uint32_t)((s1 - s0) * nkc * NTc * 128))
+                 : "memory");
+    for (int s = s0; s < s1; ++s)
+      for (int c = 0; c < nkc; ++c)
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                smem_u32(sB + (size_t)s * slice_bytes + (size_t)c * a.NT * 128)),
+            "l"(a.img + ((size_t)(s * nkc + c) * a.Np + n0) * 128), "r"((uint32_t)(NTc * 128)),
+            "r"(smem_u32(bar))
+            : "memory");
+  };
+  if (warp == kWorkers / 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+        smem_u32(&tmem_slot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    if (issuer) load_slices(0, kFirst, &bar_b[0]);
+  }
+  for (int n = tid; n < NTc; n += kThreads)
+    s_eb[n] = (unsigned short)(n0 + n < a.N ? a.eb[n0 + n] : 1);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+  // barriers, TMEM and the first digits of B overlap the previous kernel's tail
+  pdl_wait();
+  pdl_trigger();
+  if (a.done && *a.done != 0.0) {                          // uniform
+    if (issuer) wait_on(&bar_b[0], 0, &s_fail);
+    __syncthreads();
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+    return;
+  }
+
+  if (warp == kWorkers / 32) {
+    // ---- copies and MMAs: one elected lane issues (chosen by elect.sync, so
+    // that descriptors stay in uniform registers: an MMA then issues in 31
+    // clocks, its execution time, instead of 45-120 from a lane picked by its
+    // index) ----
+    __syncthreads();                                       // (the workers' exponent exchange)
+    uint32_t elected;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(elected));
+    if (issuer) load_slices(kFirst, kSlices, &bar_b[1]);
+    __syncwarp();
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t cstep = (uint32_t)(a.NT * 128) >> 4;    // descriptor steps (16 bytes)
+    const uint64_t b0 = sw128_desc(smem_u32(sB));
+    const int ksteps = a.Kp >> 4;
+    int st = 0, slices = 0;                                // slices of A known to be ready
+    bool ok = wait_on(&bar_b[0], 0, &s_fail);
+    for (int sub = 0; ok && sub < nsub; ++sub) {
+      const int nc = NTc - sub * kNS < kNS ? NTc - sub * kNS : kNS;
+      const uint32_t idesc = (1u << 4) | ((uint32_t)(nc >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
+      for (int i = 0; ok && i < per; ++i, ++st) {
+        const Step p = kStepTab[two][i];
+        if (sub == 0) {
+          for (; ok && slices <= p.g; ++slices) {
+            ok = wait_on(&bar_a[slices], 0, &s_fail);
+            if (ok && slices == kFirst) ok = wait_on(&bar_b[1], 0, &s_fail);
+          }
+        }
+        const int buf = st & 1;
+        if (ok && st >= 2) ok = wait_on(&bar_empty[buf], (uint32_t)(((st >> 1) - 1) & 1), &s_fail);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d = tm + (uint32_t)(dbase + buf * kNS);
+        if (elected) {
+          uint32_t acc = 0u;
+          for (int s = 0; s <= p.g; ++s) {
+            for (int c = p.c0; c < p.c1 && c < nkc; ++c) {
+              const uint64_t bs = b0 + (uint32_t)(((p.g - s) * slice_bytes + sub * kNS * 128) >> 4) + c * cstep;
+              const uint32_t as = tm + (uint32_t)(s * scols + c * 32);
+              const int kn = ksteps - 4 * c;
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks) {
+                if (ks < kn)
+                  asm volatile(
+                      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+                      "r"(as + (uint32_t)(ks * 8)), "l"(bs + (uint64_t)(ks * 2)), "r"(idesc), "r"(acc));
+                acc = 1u;
+              }
+            }
+          }
+          asm volatile(
+              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                  smem_u32(&bar_full[buf]))
+              : "memory");
+        }
+        __syncwarp();
+      }
+    }
+    if (!ok) s_fail = 1;
+    // the copies this warp issued land before shared memory is released
+    wait_on(&bar_b[0], 0, &s_fail);
+    wait_on(&bar_b[1], 0, &s_fail);
+  } else {
+    // ---- A: this thread's row (lane 32 q + lane) and K range [kq KQ, kq KQ + KQ) ----
+    const int q = warp & 3, kq = warp >> 2;
+    const int KQ = a.Kp >> 2;                              // 8, 16, 24 or 32
+    const int lrow = q * 32 + lane;
+    const long long m = (long long)blockIdx.x * kM + lrow;
+    const bool row_ok = m < a.M;
+    const long long hi = row_ok ? m / a.F : 0, lo = row_ok ? m - hi * a.F : 0;
+    const int k0 = kq * KQ;
+    const uint32_t lanes = (uint32_t)(q * 32) << 16;
+    int ea;
+    {
+      double x[32];
+      if (a.in_k != 1) {
+        const double *src = a.in + hi * a.in_hi + lo * a.in_lo + (long long)k0 * a.in_k;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          x[i] = (i < KQ && row_ok && k0 + i < a.K) ? __ldg(src + (long long)i * a.in_k) : 0.0;
+      } else {
+        // rows contiguous in K: a warp reads 128-byte runs of two rows at a
+        // time and transposes through its own buffer (in the part of shared
+        // memory that the later digits of B take afterwards)
+        double *buf = reinterpret_cast<double *>(sB + (size_t)kFirst * slice_bytes) + warp * 32 * 17;
+        const long long base = row_ok ? hi * a.in_hi + lo * a.in_lo : -1;
+        const int cc = lane & 15;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+          for (int t = 0; t < 16; ++t) {
+            const int k = k0 + 16 * h + cc;
+            const long long b = __shfl_sync(0xffffffffu, base, 2 * t + (lane >> 4));
+            const bool ok = b >= 0 && 16 * h + cc < KQ && k < a.K;
+            x[16 * h + t] = ok ? __ldg(a.in + b + k) : 0.0;
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          __syncwarp();
+#pragma unroll
+          for (int t = 0; t < 16; ++t) buf[(2 * t + (lane >> 4)) * 17 + cc] = x[16 * h + t];
+          __syncwarp();
+#pragma unroll
+          for (int t = 0; t < 16; ++t) x[16 * h + t] = buf[lane * 17 + t];
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
+      if (LAM && row_ok && (lane & 15) == 0) {              // the divide's table, used last
+        const double *t = a.inv_lam + hi * a.out_hi + lo * a.out_lo + (long long)n0 * a.out_n;
+        for (int n = kq; n < NTc && n0 + n < a.N; n += 4)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(t + (long long)n * a.out_n));
+      }
+      int em = 1;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) em = max(em, exp_field((uint32_t)__double2hiint(x[i])));
+      s_ea[kq][lrow] = (unsigned short)em;
+      __syncthreads();
+      ea = max(max((int)s_ea[0][lrow], (int)s_ea[1][lrow]), max((int)s_ea[2][lrow], (int)s_ea[3][lrow]));
+      uint32_t w1[32], w0[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i)
+        if (i < KQ) biased_fixed<58>(x[i], ea, w1[i], w0[i]);
+      auto put = [&](int s, auto pos, const uint32_t *w) {
+        constexpr int POS = decltype(pos)::value;
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          if (8 * b < KQ)
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                             tmem + lanes + (uint32_t)(s * scols + (k0 >> 1) + 4 * b)),
+                         "r"(digit2<POS>(w[8 * b], w[8 * b + 1])),
+                         "r"(digit2<POS>(w[8 * b + 2], w[8 * b + 3])),
+                         "r"(digit2<POS>(w[8 * b + 4], w[8 * b + 5])),
+                         "r"(digit2<POS>(w[8 * b + 6], w[8 * b + 7]))
+                         : "memory");
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_a[s]);
+      };
+      put(0, std::integral_constant<int, 2>{}, w1);
+      put(1, std::integral_constant<int, 1>{}, w1);
+      put(2, std::integral_constant<int, 0>{}, w1);
+      put(3, std::integral_constant<int, 2>{}, w0);
+      put(4, std::integral_constant<int, 1>{}, w0);
+      put(5, std::integral_constant<int, 0>{}, w0);
+    }
+    // ---- accumulators to integers, rounded once ----
+    constexpr int C = kNS / 4;                             // columns per thread in a block
+    const bool bad_row = ea == 0x7ff;
+    const long long ob = hi * a.out_hi + lo * a.out_lo;
+    int st = 0;
+    bool ok = true;
+    for (int sub = 0; ok && sub < nsub; ++sub) {
+      long long T[C];
+      for (int i = 0; i < per; ++i, ++st) {
+        const int g = kStepTab[two][i].g, buf = st & 1;
+        ok = wait_on(&bar_full[buf], (uint32_t)((st >> 1) & 1), &s_fail);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        uint32_t v[C];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+            "%14,%15}, [%16];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+              "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+            : "r"(tmem + lanes + (uint32_t)(dbase + buf * kNS + kq * C)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_empty[buf]);
+        // T in units of 2^12 of group 5: |G_0| 2^38 <= 2^62; what is dropped
+        // of groups 4 and 5 is of the order of the groups not computed
+        if (g < 4) {
+          const int wt = 1 << (28 - 10 * (g > 0 ? g - 1 : 0));
+#pragma unroll
+          for (int c = 0; c < C; ++c) {
+            const int G = __float2int_rn(__uint_as_float(v[c]));
+            T[c] = g == 0 ? (long long)G << 38 : T[c] + (long long)G * wt;
+          }
+        } else {
+          const int rs = g == 4 ? 2 : 12, half = 1 << (rs - 1);
+#pragma unroll
+          for (int c = 0; c < C; ++c)
+            T[c] += (long long)((__float2int_rn(__uint_as_float(v[c])) + half) >> rs);
+        }
+      }
+      if (!ok || !row_ok) continue;
+      const int nl0 = sub * kNS + kq * C;                  // this thread's first column, and how many
+      const int ncol = min(C, min(NTc - nl0, a.N - n0 - nl0));
+      const long long o0 = ob + (long long)(n0 + nl0) * a.out_n;
+      double lam[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) lam[c] = LAM && c < ncol ? __ldg(a.inv_lam + o0 + c * a.out_n) : 1.0;
+      bool slow = bad_row;
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        const double y = round_fixed<LAM>(T[c], ea + (int)s_eb[(nl0 + c) & (kM - 1)] - 2099, lam[c], slow);
+        if (c < ncol) a.out[o0 + c * a.out_n] = y;
+      }
+      if (slow) {                                          // rare: again, one by one
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+          if (c < ncol)
+            a.out[o0 + c * a.out_n] =
+                bad_row ? __longlong_as_double(0x7ff8000000000000ll)
+                        : round_slow(T[c], ea + (int)s_eb[nl0 + c] - 2099, lam[c]);
+      }
+    }
+    if (!ok) s_fail = 1;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (issuer && s_fail) {
+    atomicExch(a.err, (int)IGAFD_ERR_TIMEOUT);
+    // a wait ran out: give the MMAs in flight a bounded chance to finish
+    // before TMEM is released
+    const int none = 0;
+    for (int i = 0; i < 2; ++i) {
+      wait_on(&bar_full[i], 0, &none);
+      wait_on(&bar_full[i], 1, &none);
+    }
+  }
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+}
+
+// Digits of B = U_k^T (transpose) or U_k as the shared-memory images of the
+// pass kernel, and the exponent field of each row: one CTA per (row, image).
+struct ImgJob {
+  const double *U;
+  int n, Np, Kp, transpose;
+  unsigned char *img;
+  int *eb;
+};
+struct ImgBatch {
+  ImgJob j[6];
+};
+__global__ void __launch_bounds__(128) split_image_kernel(ImgBatch b) {
+  const ImgJob J = b.j[blockIdx.y];
+  const int r = blockIdx.x, k = threadIdx.x;
+  if (r >= J.Np) return;
+  __shared__ int s_e[4];
+  const int nkc = (J.Kp + 63) >> 6;
+  double d = 0.0;
+  if (r < J.n && k < J.n) d = J.transpose ? J.U[(size_t)k * J.n + r] : J.U[(size_t)r * J.n + k];
+  int e = exp_field((uint32_t)__double2hiint(d));
+  for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+  if ((k & 31) == 0) s_e[k >> 5] = e;
+  __syncthreads();
+  e = max(max(s_e[0], s_e[1]), max(s_e[2], s_e[3]));
+  if (k == 0) J.eb[r] = e;
+  if (k >= nkc * 64) return;
+  uint32_t w1, w0;
+  biased_fixed<59>(d, e, w1, w0);
+  const int kb = (k & 63) * 2;
+  unsigned char *at = J.img + ((size_t)(k >> 6) * J.Np + r) * 128 + ((((kb >> 4) ^ (r & 7)) << 4) | (kb & 15));
+  const size_t slice = (size_t)nkc * J.Np * 128;
+  auto put = [&](int s, uint32_t w) { *reinterpret_cast<unsigned short *>(at + s * slice) = (unsigned short)w; };
+  put(0, __half_as_ushort(__int2half_rn((int)(w1 >> 20) - 512)));   // -512..512
+  put(1, digit2<1>(w1, w1));
+  put(2, digit2<0>(w1, w1));
+  put(3, digit2<2>(w0, w0));
+  put(4, digit2<1>(w0, w0));
+  put(5, digit2<0>(w0, w0));
+}
+
+int pad(int n, int to) { return (n + to - 1) / to * to; }
+
+size_t pass_smem(int Kp, int NT) {
+  const size_t slice = (size_t)((Kp + 63) / 64) * NT * 128;
+  const size_t a = kSlices * slice, b = kFirst * slice + kTrans;
+  return 1024 + (a > b ? a : b);
+}
+
+}  // namespace
+
+struct FDSplit {
+  unsigned char *img[3][2];   // [direction][0: U_k^T, 1: U_k]
+  int *eb[3][2];
+};
+
+bool igafd_fd_split_shape(const igafd_patch *P) {
+  for (int k = 0; k < P->dim; ++k)
+    if (P->n[k] > 128) return false;
+  return true;
+}
+
+// Digit images of U_k^T and U_k. Allocates on the first call; later calls (a
+// re-setup of P) refill the same buffers. Enqueues one kernel.
+igafd_status igafd_fd_split_init(igafd_patch *P, cudaStream_t s) {
+  if (!igafd_fd_split_shape(P)) return IGAFD_OK;
+  if (!P->split) {
+    P->split = (FDSplit *)calloc(1, sizeof(FDSplit));
+    if (!P->split) return IGAFD_ERR_OOM;
+  }
+  ImgBatch b{};
+  int jobs = 0, rows = 0;
+  for (int k = 0; k < P->dim; ++k)
+    for (int d = 0; d < 2; ++d) {
+      ImgJob &J = b.j[jobs++];
+      J.U = P->U[k]; J.n = P->n[k]; J.Np = pad(P->n[k], 16); J.Kp = pad(P->n[k], 32);
+      J.transpose = d == 0;
+      const size_t sz = (size_t)kSlices * ((J.Kp + 63) / 64) * J.Np * 128;
+      if ((!P->split->img[k][d] && cudaMalloc(&P->split->img[k][d], sz) != cudaSuccess) ||
+          (!P->split->eb[k][d] && cudaMalloc(&P->split->eb[k][d], J.Np * sizeof(int)) != cudaSuccess)) {
+        cudaGetLastError();
+        return IGAFD_ERR_OOM;
+      }
+      J.img = P->split->img[k][d];
+      J.eb = P->split->eb[k][d];
+      rows = J.Np > rows ? J.Np : rows;
+    }
+  split_image_kernel<<<dim3(rows, jobs), 128, 0, s>>>(b);
+  IGAFD_LAUNCHED(1);
+  IGAFD_CUDA(cudaGetLastError());
+  return IGAFD_OK;
+}
+
+void igafd_fd_split_free(igafd_patch *P) {
+  if (!P || !P->split) return;
+  for (int k = 0; k < 3; ++k)
+    for (int d = 0; d < 2; ++d) {
+      cudaFree(P->split->img[k][d]);
+      cudaFree(P->split->eb[k][d]);
+    }
+  free(P->split);
+  P->split = nullptr;
+}
+
+// One mode product: rows m = hi F + lo at in + hi in_hi + lo in_lo + k in_k.
+static igafd_status launch_pass(igafd_patch *P, int k, int dir, SplitArgs a, cudaStream_t s) {
+  a.K = a.N = P->n[k];
+  a.Kp = pad(a.K, 32);
+  a.Np = pad(a.N, 16);
+  a.img = P->split->img[k][dir];
+  a.eb = P->split->eb[k][dir];
+  a.err = P->err_flag;
+  // Column split: with fewer 128-row tiles than SMs, a CTA's columns are
+  // halved while all CTAs still fit one wave (a CTA's time is about half the
+  // splitting of its rows, which every column part repeats, and half the
+  // digit products, which shrink with the columns).
+  const long long tiles = (a.M + kM - 1) / kM;
+  int parts = 1;
+  while (parts < 8 && tiles * parts * 2 <= P->num_sms && pad(a.Np, 32 * parts) / parts > 16) parts *= 2;
+  a.NT = pad((a.Np + parts - 1) / parts, 16);
+  parts = (a.Np + a.NT - 1) / a.NT;
+  const size_t smem = pass_smem(a.Kp, a.NT);
+  static std::atomic<unsigned long long> attr_set{0};
+  const unsigned long long bit = 1ull << (P->dev & 63);
+  if (!(attr_set.load() & bit)) {
+    for (auto kern : {split_pass_kernel<false>, split_pass_kernel<true>})
+      IGAFD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)pass_smem(128, 128)));
+    attr_set.fetch_or(bit);
+  }
+  IGAFD_CUDA(igafd_launch(a.inv_lam ? split_pass_kernel<true> : split_pass_kernel<false>,
+                          dim3((unsigned)tiles, (unsigned)parts), dim3(kThreads), smem, s, a));
+  IGAFD_LAUNCHED(1);
+  return IGAFD_OK;
+}
+
+// z = P^{-1} r. 3D: [i3][i2][i1] -> [j3][i2][i1] -> [j3][j2][i1] ->
+// [j1][j3][j2] (divided) -> [i1][j3][j2] -> [i1][i3][j2] -> [i3][i2][i1];
+// 2D: [i2][i1] -> [j2][i1] -> [j1][j2] (divided) -> [i1][j2] -> [i2][i1].
+igafd_status igafd_fd_split_apply(igafd_patch *P, const double *r, double *z, cudaStream_t s,
+                                  double *done_flag) {
+  if (!P->split) return IGAFD_ERR_ARG;
+  const long long n1 = P->n[0], n2 = P->n[1], n3 = P->dim == 3 ? P->n[2] : 1;
+  const long long n12 = n1 * n2, n23 = n2 * n3;
+  double *t1 = P->fd_a, *t2 = P->fd_b;
+  SplitArgs a{};
+  a.done = done_flag;
+  auto pass = [&](int k, int dir, const double *in, double *out, long long M, long long F,
+                  long long in_hi, long long in_lo, long long in_k, long long out_hi,
+                  long long out_lo, long long out_n, const double *inv_lam) {
+    a.in = in; a.out = out; a.M = M; a.F = (int)F;
+    a.in_hi = in_hi; a.in_lo = in_lo; a.in_k = in_k;
+    a.out_hi = out_hi; a.out_lo = out_lo; a.out_n = out_n;
+    a.inv_lam = inv_lam;
+    return launch_pass(P, k, dir, a, s);
+  };
+  if (P->dim == 3) {
+    IGAFD_TRY(pass(2, 0, r, t1, n12, n12, 0, 1, n12, 0, 1, n12, nullptr));
+    IGAFD_TRY(pass(1, 0, t1, t2, n1 * n3, n1, n12, 1, n1, n12, 1, n1, nullptr));
+    IGAFD_TRY(pass(0, 0, t2, t1, n23, n23, 0, n1, 1, 0, 1, n23, P->inv_lam));
+    IGAFD_TRY(pass(0, 1, t1, t2, n23, n23, 0, 1, n23, 0, 1, n23, nullptr));
+    IGAFD_TRY(pass(2, 1, t2, t1, n12, n2, n23, 1, n2, n23, 1, n2, nullptr));
+    // rows m = i3 n1 + i1 of [i1][i3][j2], contiguous in j2
+    return pass(1, 1, t1, z, n1 * n3, n1, n2, n23, 1, n12, 1, n1, nullptr);
+  }
+  IGAFD_TRY(pass(1, 0, r, t1, n1, n1, 0, 1, n1, 0, 1, n1, nullptr));
+  IGAFD_TRY(pass(0, 0, t1, t2, n2, n2, 0, n1, 1, 0, 1, n2, P->inv_lam));
+  IGAFD_TRY(pass(0, 1, t2, t1, n2, n2, 0, 1, n2, 0, 1, n2, nullptr));
+  return pass(1, 1, t1, z, n1, n1, 0, n2, 1, 0, 1, n1, nullptr);
+}
