@@ -163,6 +163,9 @@ igafd_status igafd_build_prec(igafd_patch *P, cudaStream_t s);
 igafd_status igafd_setup_pencils_eig(igafd_patch *P, cudaStream_t s, const double *const *wK = nullptr,
                                      const double *const *wM = nullptr);
 igafd_status igafd_setup_stencil(igafd_patch *P, cudaStream_t s);
+// 3D (assemble3.cu): geometry diagnostics and stencil; b += the load vector
+igafd_status igafd_assemble3(igafd_patch *P, cudaStream_t s);
+igafd_status igafd_load3(igafd_patch *P, const double *fq, double *b, cudaStream_t s);
 // a half-stored stencil written out in the full layout [n_off][N] (setup.cu)
 igafd_status igafd_stencil_expand(const igafd_patch *P, double *dst, cudaStream_t s);
 // dense (Dirichlet-reduced) pencils K_k, M_k of direction k into K, M (n_k x
