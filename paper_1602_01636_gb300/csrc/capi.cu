@@ -91,6 +91,14 @@ igafd_status build(igafd_patch *P, const igafd_patch_desc *d, cudaStream_t s) {
   IGAFD_TRY(alloc(&P->inv_lam, (size_t)N));
   IGAFD_TRY(alloc(&P->inv_lam32, (size_t)N));
   P->Np = igafd_stencil_row_stride(N);
+  // Stencil pipeline until the autotuner or the caller picks one. Ring depth:
+  // the most that still leaves three CTAs per SM (a stage holds 2p + 1 runs):
+  // at n = 64, p = 2 depths 3 / 4 / 6 took 69 / 63 / 61 us, at p = 3 163 / 155 /
+  // 165, at p = 4 319 / 336 / 404. Two rows per thread only where every SM has
+  // many tiles (n = 128, p = 3: 1.177 against 1.194 ms with one; n = 64: 158
+  // against 155 us).
+  P->stencil_stages = P->dim == 2 || P->p == 3 ? 4 : P->p < 3 ? 6 : 3;
+  P->stencil_rows = P->dim == 3 && N >= (1ll << 20) ? 2 : 1;
   const bool with_stencil = !(d->flags & IGAFD_SETUP_NO_STENCIL);
   P->stencil_half = (d->flags & IGAFD_SETUP_HALF_STENCIL) ? 1 : 0;
   if (P->stencil_half) {
@@ -212,7 +220,6 @@ extern "C" igafd_status igafd_setup_patch(const igafd_patch_desc *d, void *strea
   P->kappa = d->kappa;
   P->fd_fused = 1;
   for (int o = 0; o < 3; ++o) P->fd_fused_op[o] = 1;
-  P->stencil_rows = 1;
   if (cudaGetDevice(&P->dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, P->dev) != cudaSuccess) {
     free(P);

@@ -33,11 +33,11 @@ __global__ void __launch_bounds__(kTile / R + 32) stencil_tma_kernel(StencilArgs
                                               &s_abort);
 }
 
-// One launch of the single-problem kernel, or with grid_out only its grid
-// (the resident CTAs of every SM, at most grid_cap).
+// One launch of the single-problem kernel (the resident CTAs of every SM, at
+// most one per tile and one per partial sum), or with grid_out only its grid
+// and tiles.
 template <int DIM, int P, int MODE, int kStages, int R, bool HALF = false>
-igafd_status launch_one(const StencilArgs &a, long long grid_cap, int num_sms, cudaStream_t s,
-                        long long *grid_out) {
+igafd_status launch_one(StencilArgs &a, int num_sms, cudaStream_t s, long long *grid_out) {
   const size_t smem =
       (size_t)kStages * Geom<P, HALF>::STAGE * sizeof(double) + 2 * kStages * sizeof(uint64_t);
   constexpr int kBlock = kTile / R + 32;
@@ -46,9 +46,11 @@ igafd_status launch_one(const StencilArgs &a, long long grid_cap, int num_sms, c
   static std::atomic<int> per_sm_tab[64];
   int per_sm = 1;
   IGAFD_TRY(per_sm_of(kern, kBlock, smem, attr_set, per_sm_tab, &per_sm));
+  a.tile = tile_rows(a.N, num_sms, per_sm, 32 * R);
+  a.ntiles = (a.N + a.tile - 1) / a.tile;
   long long grid = (long long)num_sms * per_sm;
-  if (grid > grid_cap) grid = grid_cap;
-  if (grid < 1) grid = 1;
+  if (grid > a.ntiles) grid = a.ntiles;
+  if (grid > IGAFD_RED_BLOCKS) grid = IGAFD_RED_BLOCKS;
   if (grid_out) {
     *grid_out = grid;
     return IGAFD_OK;
@@ -60,44 +62,42 @@ igafd_status launch_one(const StencilArgs &a, long long grid_cap, int num_sms, c
 
 // two rows per thread are built for 3D only (2D patches are small)
 template <int DIM, int P, int MODE, int kStages>
-igafd_status launch_rows(int rows, const StencilArgs &a, long long cap, int sms, cudaStream_t s,
-                         long long *grid_out) {
+igafd_status launch_rows(int rows, StencilArgs &a, int sms, cudaStream_t s, long long *grid_out) {
   if constexpr (DIM == 3)
-    if (rows == 2) return launch_one<DIM, P, MODE, kStages, 2>(a, cap, sms, s, grid_out);
-  return launch_one<DIM, P, MODE, kStages, 1>(a, cap, sms, s, grid_out);
+    if (rows == 2) return launch_one<DIM, P, MODE, kStages, 2>(a, sms, s, grid_out);
+  return launch_one<DIM, P, MODE, kStages, 1>(a, sms, s, grid_out);
 }
 
 // a half-stored stencil runs at the default ring depth
 template <int DIM, int P, int MODE>
-igafd_status launch_half(int rows, const StencilArgs &a, long long cap, int sms, cudaStream_t s,
-                         long long *grid_out) {
+igafd_status launch_half(int rows, StencilArgs &a, int sms, cudaStream_t s, long long *grid_out) {
   if constexpr (DIM == 3)
-    if (rows == 2) return launch_one<DIM, P, MODE, kStagesDefault, 2, true>(a, cap, sms, s, grid_out);
-  return launch_one<DIM, P, MODE, kStagesDefault, 1, true>(a, cap, sms, s, grid_out);
+    if (rows == 2) return launch_one<DIM, P, MODE, kStagesDefault, 2, true>(a, sms, s, grid_out);
+  return launch_one<DIM, P, MODE, kStagesDefault, 1, true>(a, sms, s, grid_out);
 }
 
 template <int DIM, int P, int MODE>
-igafd_status launch_stages(int stages, int rows, const StencilArgs &a, long long cap, int sms,
-                           cudaStream_t s, long long *grid_out) {
-  if (stages < 0) return launch_half<DIM, P, MODE>(rows, a, cap, sms, s, grid_out);
+igafd_status launch_stages(int stages, int rows, StencilArgs &a, int sms, cudaStream_t s,
+                           long long *grid_out) {
+  if (stages < 0) return launch_half<DIM, P, MODE>(rows, a, sms, s, grid_out);
   switch (stages) {
-    case 3: return launch_rows<DIM, P, MODE, 3>(rows, a, cap, sms, s, grid_out);
-    case 6: return launch_rows<DIM, P, MODE, 6>(rows, a, cap, sms, s, grid_out);
-    default: return launch_rows<DIM, P, MODE, 4>(rows, a, cap, sms, s, grid_out);
+    case 3: return launch_rows<DIM, P, MODE, 3>(rows, a, sms, s, grid_out);
+    case 6: return launch_rows<DIM, P, MODE, 6>(rows, a, sms, s, grid_out);
+    default: return launch_rows<DIM, P, MODE, 4>(rows, a, sms, s, grid_out);
   }
 }
 
 template <int DIM, int MODE>
-igafd_status launch_p(int p, int stages, int rows, const StencilArgs &a, long long cap, int sms,
-                      cudaStream_t s, long long *grid_out = nullptr) {
+igafd_status launch_p(int p, int stages, int rows, StencilArgs &a, int sms, cudaStream_t s,
+                      long long *grid_out = nullptr) {
   switch (p) {
-    case 1: return launch_stages<DIM, 1, MODE>(stages, rows, a, cap, sms, s, grid_out);
-    case 2: return launch_stages<DIM, 2, MODE>(stages, rows, a, cap, sms, s, grid_out);
-    case 3: return launch_stages<DIM, 3, MODE>(stages, rows, a, cap, sms, s, grid_out);
-    case 4: return launch_stages<DIM, 4, MODE>(stages, rows, a, cap, sms, s, grid_out);
-    case 5: return launch_stages<DIM, 5, MODE>(stages, rows, a, cap, sms, s, grid_out);
-    case 6: return launch_stages<DIM, 6, MODE>(stages, rows, a, cap, sms, s, grid_out);
-    case 7: return launch_stages<DIM, 7, MODE>(stages, rows, a, cap, sms, s, grid_out);
+    case 1: return launch_stages<DIM, 1, MODE>(stages, rows, a, sms, s, grid_out);
+    case 2: return launch_stages<DIM, 2, MODE>(stages, rows, a, sms, s, grid_out);
+    case 3: return launch_stages<DIM, 3, MODE>(stages, rows, a, sms, s, grid_out);
+    case 4: return launch_stages<DIM, 4, MODE>(stages, rows, a, sms, s, grid_out);
+    case 5: return launch_stages<DIM, 5, MODE>(stages, rows, a, sms, s, grid_out);
+    case 6: return launch_stages<DIM, 6, MODE>(stages, rows, a, sms, s, grid_out);
+    case 7: return launch_stages<DIM, 7, MODE>(stages, rows, a, sms, s, grid_out);
     default: return IGAFD_ERR_ARG;
   }
 }
@@ -133,7 +133,7 @@ static StencilArgs make_args(igafd_patch *P, const double *x, double *y, const d
   a.Np = P->stencil_half ? P->sh_ld : P->Np;
   a.oc = P->stencil_half ? P->n_off / 2 : 0;
   a.shH = P->stencil_half ? P->sh_H : 0;
-  a.ntiles = (P->N + kTile - 1) / kTile;
+  a.pad = P->Np;
   a.partial = pcg ? P->partial : nullptr;
   a.counter = P->counter;
   a.scal = pcg ? P->scal : nullptr;
@@ -145,11 +145,6 @@ static StencilArgs make_args(igafd_patch *P, const double *x, double *y, const d
   return a;
 }
 
-static long long grid_cap(igafd_patch *P) {
-  const long long ntiles = (P->N + kTile - 1) / kTile;
-  return ntiles < IGAFD_RED_BLOCKS ? ntiles : IGAFD_RED_BLOCKS;
-}
-
 igafd_status igafd_stencil_launch(igafd_patch *P, const double *x, double *y, const double *b,
                                   int pcg, int skip_done, cudaStream_t s, int every,
                                   unsigned long long *tstat, const double *z) {
@@ -159,19 +154,16 @@ igafd_status igafd_stencil_launch(igafd_patch *P, const double *x, double *y, co
     IGAFD_CUDA(cudaMemcpyAsync(P->xpad, x, P->N * sizeof(double), cudaMemcpyDeviceToDevice, s));
     x = P->xpad;
   }
-  const StencilArgs a = make_args(P, x, y, b, pcg, skip_done, every, tstat, z);
-  // persistent grid: the resident CTAs of every SM, never more than the
-  // tiles or the partial-sum slots
-  const long long cap = grid_cap(P);
+  StencilArgs a = make_args(P, x, y, b, pcg, skip_done, every, tstat, z);
   // ring depth; -1 selects the half-stored stencil's kernels (default depth)
   const int st = P->stencil_half ? -1 : P->stencil_stages > 0 ? P->stencil_stages : kStagesDefault;
   const int rows = P->stencil_rows == 2 ? 2 : 1;
   if (P->dim == 3) {
-    if (b) return launch_p<3, 1>(P->p, st, rows, a, cap, P->num_sms, s);
-    return launch_p<3, 0>(P->p, st, rows, a, cap, P->num_sms, s);
+    if (b) return launch_p<3, 1>(P->p, st, rows, a, P->num_sms, s);
+    return launch_p<3, 0>(P->p, st, rows, a, P->num_sms, s);
   }
-  if (b) return launch_p<2, 1>(P->p, st, 1, a, cap, P->num_sms, s);
-  return launch_p<2, 0>(P->p, st, 1, a, cap, P->num_sms, s);
+  if (b) return launch_p<2, 1>(P->p, st, 1, a, P->num_sms, s);
+  return launch_p<2, 0>(P->p, st, 1, a, P->num_sms, s);
 }
 
 // ---- for the batched solve -------------------------------------------------
@@ -183,18 +175,19 @@ size_t igafd_stencil_args_bytes() { return sizeof(StencilArgs); }
 // whose CTAs a batched launch runs as work items.
 igafd_status igafd_stencil_batch_args(igafd_patch *P, int sel, int flexible, int every, void *out,
                                       long long *vgrid) {
-  const StencilArgs a = sel == 0 ? make_args(P, P->pv, P->q, nullptr, 1, 0, 0, nullptr, nullptr)
-                                 : make_args(P, P->xs, P->r, P->bint, 1, 0, sel == 1 ? every : 0,
-                                             nullptr, flexible ? P->z : nullptr);
-  memcpy(out, &a, sizeof(a));
-  const long long cap = grid_cap(P);
+  StencilArgs a = sel == 0 ? make_args(P, P->pv, P->q, nullptr, 1, 0, 0, nullptr, nullptr)
+                           : make_args(P, P->xs, P->r, P->bint, 1, 0, sel == 1 ? every : 0, nullptr,
+                                       flexible ? P->z : nullptr);
   // ring depth; -1 selects the half-stored stencil's kernels (default depth)
   const int st = P->stencil_half ? -1 : P->stencil_stages > 0 ? P->stencil_stages : kStagesDefault;
   const int rows = P->dim == 3 && P->stencil_rows == 2 ? 2 : 1;
-  if (P->dim == 3) {
-    if (sel) return launch_p<3, 1>(P->p, st, rows, a, cap, P->num_sms, nullptr, vgrid);
-    return launch_p<3, 0>(P->p, st, rows, a, cap, P->num_sms, nullptr, vgrid);
-  }
-  if (sel) return launch_p<2, 1>(P->p, st, 1, a, cap, P->num_sms, nullptr, vgrid);
-  return launch_p<2, 0>(P->p, st, 1, a, cap, P->num_sms, nullptr, vgrid);
+  igafd_status status;
+  if (P->dim == 3)
+    status = sel ? launch_p<3, 1>(P->p, st, rows, a, P->num_sms, nullptr, vgrid)
+                 : launch_p<3, 0>(P->p, st, rows, a, P->num_sms, nullptr, vgrid);
+  else
+    status = sel ? launch_p<2, 1>(P->p, st, 1, a, P->num_sms, nullptr, vgrid)
+                 : launch_p<2, 0>(P->p, st, 1, a, P->num_sms, nullptr, vgrid);
+  memcpy(out, &a, sizeof(a));
+  return status;
 }

@@ -27,7 +27,7 @@
 
 namespace {
 
-constexpr int kTile = 256;                        // rows per tile
+constexpr int kTile = 256;                        // rows per tile at most (StencilArgs::tile in use)
 // ring depths (offset groups in flight per CTA) the kernel is built for; the
 // autotuner picks one per (dimension, degree, sizes), default kStagesDefault
 constexpr int kStagesDefault = 4;
@@ -101,6 +101,8 @@ struct StencilArgs {
   const double *z;    // MODE 1, optional: also (y, z) -> scal[S_RZOLD] (flexible beta)
   int n1, n2, n3;
   long long N, Np;
+  long long pad;      // rows the stencil arrays hold (N rounded up to kTile)
+  int tile;           // rows per tile (a multiple of 64 with two rows per thread, else of 32)
   long long ntiles;
   double *partial;    // null: no dot
   unsigned *counter;
@@ -167,14 +169,20 @@ __device__ __forceinline__ void stencil_cta(const StencilArgs &a, long long vb, 
   constexpr int RS = Gm::RS;
   constexpr int NOFF = DIM == 3 ? W * W * W : W * W;
   constexpr int G = DIM == 3 ? W * W : W;        // (delta_2, delta_3) groups per tile
-  constexpr uint32_t kStageBytes = Gm::STAGE * sizeof(double);
   constexpr int kCompute = kTile / R;            // compute threads
+  constexpr int NV = ((W + 1) / 2 + 1) * 2;      // x values a two-row thread holds
   static_assert(R == 1 || R == 2, "one or two rows per thread");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long my_tiles = a.ntiles > vb ? (a.ntiles - 1 - vb) / vgrid + 1 : 0;
-  const long long total = my_tiles * G;
+  const int my_tiles = (int)(a.ntiles > vb ? (a.ntiles - 1 - vb) / vgrid + 1 : 0);
+  const long long total = (long long)my_tiles * G;
   const long long n12 = (long long)a.n1 * a.n2;
   const long long g0 = gstage;                   // global index of this call's first stage
+  const int h = a.tile;
+  // ring position, advanced step by step (a step: one (delta_2, delta_3)
+  // group of one tile): slot, and how often the ring has come round
+  int slot = (int)(g0 % kStages);
+  uint32_t turn = (uint32_t)(g0 / kStages);
+  constexpr int D3 = DIM == 3 ? W : 1;           // delta_3 values
 
   double dot = 0.0, dot2 = 0.0;
   if (warp == kCompute / 32) {
@@ -182,47 +190,54 @@ __device__ __forceinline__ void stencil_cta(const StencilArgs &a, long long vb, 
     if (lane == 0) {
       long long issued = 0;
       bool ok = true;
-      for (long long s = 0; s < total && ok; ++s) {
-        const long long gs = g0 + s;
-        const int slot = (int)(gs % kStages);
-        if (gs >= kStages) {
-          const uint32_t par = (uint32_t)(((gs / kStages) - 1) & 1);
-          long long it = 0;
-          while (!mbar_try_wait(&empty[slot], par)) {
-            if (*s_abort || ++it > kSpin) { ok = false; break; }
-          }
-          if (!ok) break;
-        }
-        const long long tile = vb + (s / G) * vgrid;
-        const int g = (int)(s % G);
-        const int d2 = g % W - P, d3 = DIM == 3 ? g / W - P : 0;
-        const int ob = (DIM == 3 ? (d3 + P) * W * W : 0) + (d2 + P) * W;
-        const long long row0 = tile * kTile;
-        long long x0 = row0 + (long long)d3 * n12 + (long long)d2 * a.n1 - P;
-        x0 -= (x0 & 1);                                   // 16-byte aligned start
-        double *st = ring + (size_t)slot * Gm::STAGE;
-        uint64_t *bar = &full[slot];
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive_tx(bar, kStageBytes);
-        if constexpr (!HALF) {
-          for (int d1 = 0; d1 < W; ++d1)
-            bulk_g2s(st + d1 * kTile, a.S + (size_t)(ob + d1) * a.Np + row0, kTile * sizeof(double),
-                     bar);
-        } else {
-          for (int d1 = 0; d1 < W; ++d1) {
-            const int o = ob + d1;
-            long long start = a.shH + row0;
-            int arr = o - a.oc;
-            if (o < a.oc) {                                 // delta < 0: the mirrored run
-              arr = NOFF - 1 - o - a.oc;
-              start += (d1 - P) + (long long)d2 * a.n1 + (long long)d3 * n12;
+      const uint32_t xrun = (uint32_t)(((h + 2 * P + 3) & ~1) * sizeof(double));
+      long long row0 = vb * h;
+      for (int t = 0; t < my_tiles && ok; ++t, row0 += vgrid * h) {
+        // the last tile's rows end with the arrays (both multiples of 32)
+        const int rows = (int)(a.pad - row0 < h ? a.pad - row0 : h);
+        const uint32_t run = (uint32_t)((HALF ? rows + 2 : rows) * sizeof(double));
+        int ob = 0;                                        // first offset of the group
+#pragma unroll 1
+        for (int d3 = 0; d3 < D3 && ok; ++d3) {
+          const long long off3 = DIM == 3 ? (d3 - P) * n12 : 0;
+#pragma unroll 1
+          for (int d2 = 0; d2 < W; ++d2, ob += W) {
+            if (turn > 0) {
+              long long it = 0;
+              while (!mbar_try_wait(&empty[slot], (turn - 1) & 1)) {
+                if (*s_abort || ++it > kSpin) { ok = false; break; }
+              }
+              if (!ok) break;
             }
-            start -= (start & 1);
-            bulk_g2s(st + d1 * RS, a.S + (size_t)arr * a.Np + start, RS * sizeof(double), bar);
+            const long long off23 = off3 + (long long)(d2 - P) * a.n1;
+            long long x0 = row0 + off23 - P;
+            x0 -= (x0 & 1);                                // 16-byte aligned start
+            double *st = ring + (size_t)slot * Gm::STAGE;
+            uint64_t *bar = &full[slot];
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive_tx(bar, W * run + xrun);
+            if constexpr (!HALF) {
+              const double *src = a.S + (size_t)ob * a.Np + row0;
+#pragma unroll
+              for (int d1 = 0; d1 < W; ++d1) bulk_g2s(st + d1 * kTile, src + (size_t)d1 * a.Np, run, bar);
+            } else {
+              for (int d1 = 0; d1 < W; ++d1) {
+                const int o = ob + d1;
+                long long start = a.shH + row0;
+                int arr = o - a.oc;
+                if (o < a.oc) {                            // delta < 0: the mirrored run
+                  arr = NOFF - 1 - o - a.oc;
+                  start += (d1 - P) + off23;
+                }
+                start -= (start & 1);
+                bulk_g2s(st + d1 * RS, a.S + (size_t)arr * a.Np + start, run, bar);
+              }
+            }
+            bulk_g2s(st + W * RS, a.x + x0, xrun, bar);
+            ++issued;
+            if (++slot == kStages) { slot = 0; ++turn; }
           }
         }
-        bulk_g2s(st + W * RS, a.x + x0, Gm::XW * sizeof(double), bar);
-        ++issued;
       }
       if (!ok) {
         *s_abort = 1;
@@ -234,135 +249,141 @@ __device__ __forceinline__ void stencil_cta(const StencilArgs &a, long long vb, 
     }
   } else {
     // ---------------- compute warps ----------------
-    double acc[R];
+    // Two accumulators per row (even and odd offsets of a run): the FMA
+    // chains of a warp are then short enough that a CTA alone on its SM (the
+    // last tiles, small patches) is not held up by the FMA latency.
+    bool ok = true;
+    const int t0 = R * tid;                      // first of this thread's R rows in the tile
+    long long row0 = vb * h;
+    for (int t = 0; t < my_tiles && ok; ++t, row0 += vgrid * h) {
+      const long long row = row0 + t0;
+      double acc[R][2];
+      bool live[R];
+      // bit d of v2, v3: (i_2 + d - P, i_3 + d' - P) inside the box
+      uint32_t v2[R], v3[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = 0.0;
-    long long row = 0;                       // first of this thread's R rows
-    bool live[R];
-    int i2r[R], i3r[R];
+      for (int r = 0; r < R; ++r) {
+        acc[r][0] = acc[r][1] = 0.0;
+        live[r] = t0 + r < h && row + r < a.N;
+        const uint32_t j = (uint32_t)(row + r) / (uint32_t)a.n1;
+        const int i2 = (int)(j % (uint32_t)a.n2), i3 = DIM == 3 ? (int)(j / (uint32_t)a.n2) : 0;
+        v2[r] = v3[r] = 0u;
 #pragma unroll
-    for (int r = 0; r < R; ++r) { live[r] = false; i2r[r] = 0; i3r[r] = 0; }
-    for (long long s = 0; s < total; ++s) {
-      const int g = (int)(s % G);
-      if (g == 0) {
-        const long long tile = vb + (s / G) * vgrid;
-        row = tile * kTile + (long long)R * tid;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          live[r] = row + r < a.N;
-          i2r[r] = (int)(((row + r) / a.n1) % a.n2);
-          i3r[r] = DIM == 3 ? (int)((row + r) / n12) : 0;
-          acc[r] = 0.0;
+        for (int d = 0; d < W; ++d) {
+          if (live[r] && (unsigned)(i2 + d - P) < (unsigned)a.n2) v2[r] |= 1u << d;
+          if (live[r] && (DIM == 2 || (unsigned)(i3 + d - P) < (unsigned)a.n3)) v3[r] |= 1u << d;
         }
       }
-      const long long gs = g0 + s;
-      const int slot = (int)(gs % kStages);
-      const uint32_t par = (uint32_t)((gs / kStages) & 1);
-      long long it = 0;
-      bool ok = true;
-      while (!mbar_try_wait(&full[slot], par)) {
-        if (*s_abort || ++it > kSpin) { ok = false; break; }
-      }
-      if (!ok) {
-        *s_abort = 1;
-        atomicExch(a.err, (int)IGAFD_ERR_TIMEOUT);
-        break;
-      }
-      const int d2 = g % W - P, d3 = DIM == 3 ? g / W - P : 0;
-      const long long row0 = row - (long long)R * tid;
-      const long long xs0 = row0 + (long long)d3 * n12 + (long long)d2 * a.n1 - P;
-      const int sh = (int)(xs0 & 1);                      // window starts at xs0 - sh
-      const double *st = ring + (size_t)slot * Gm::STAGE;
-      // rows whose (i_2 + delta_2, i_3 + delta_3) leaves the box have only
-      // zero coefficients in this group; skip when the whole warp is out
-      bool in23 = false;
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        in23 = in23 || (live[r] && (i2r[r] + d2 >= 0) && (i2r[r] + d2 < a.n2) &&
-                        (DIM == 2 || ((i3r[r] + d3 >= 0) && (i3r[r] + d3 < a.n3))));
-      // HALF: run j of this group starts one row late when it is mirrored and
-      // its start row was odd
-      int hs[W];
-#pragma unroll
-      for (int j = 0; j < W; ++j) hs[j] = 0;
-      if constexpr (HALF) {
-        const int ob = (DIM == 3 ? (d3 + P) * W * W : 0) + (d2 + P) * W;
-        const long long pb = a.shH + row0 + (long long)d2 * a.n1 + (long long)d3 * n12 - P;
-#pragma unroll
-        for (int j = 0; j < W; ++j) hs[j] = ob + j < a.oc ? (int)((pb + j) & 1) : 0;
-      }
-      if (__any_sync(0xffffffffu, in23)) {
-        if constexpr (R == 1) {
-          const double *cf = st + tid;
-          const double *xw = st + W * RS + tid + sh;      // xw[j] = x[row + off - P + j]
-#pragma unroll
-          for (int j = 0; j < W; ++j) acc[0] = fma(cf[j * RS + hs[j]], xw[j], acc[0]);
-        } else if constexpr (HALF) {
-          // rows row, row + 1: coefficients st[j RS + 2 tid + hs[j]] and the next;
-          // x[row + off - P + j] = xv[j + sh], x[row + 1 + off - P + j] = xv[j + 1 + sh]
-          const double *cf = st + 2 * tid;
-          const double2 *xb = reinterpret_cast<const double2 *>(st + W * RS + 2 * tid);
-          constexpr int NP = (W + 1) / 2;
-          double xv[2 * NP + 2];
-#pragma unroll
-          for (int m = 0; m < NP + 1; ++m) { const double2 v = xb[m]; xv[2 * m] = v.x; xv[2 * m + 1] = v.y; }
-          // two 8-byte loads per run (no branch on the shift, so all of the
-          // group's loads issue together)
-          double c0[W], c1[W];
-#pragma unroll
-          for (int j = 0; j < W; ++j) {
-            c0[j] = cf[j * RS + hs[j]];
-            c1[j] = cf[j * RS + hs[j] + 1];
+      const int odd0 = (int)((row0 - P) & 1), odd1 = a.n1 & 1, odd12 = (int)(n12 & 1);
+      int ob = 0;
+#pragma unroll 1
+      for (int d3 = 0; d3 < D3 && ok; ++d3) {
+#pragma unroll 1
+        for (int d2 = 0; d2 < W; ++d2, ob += W) {
+          long long it = 0;
+          while (!mbar_try_wait(&full[slot], turn & 1)) {
+            if (*s_abort || ++it > kSpin) { ok = false; break; }
           }
-#pragma unroll
-          for (int j = 0; j < W; ++j) {
-            acc[0] = fma(c0[j], xv[j + sh], acc[0]);
-            acc[1] = fma(c1[j], xv[j + 1 + sh], acc[1]);
+          if (!ok) {
+            *s_abort = 1;
+            atomicExch(a.err, (int)IGAFD_ERR_TIMEOUT);
+            break;
           }
+          // the x window starts sh elements before row0 + off(0, d2, d3) - P
+          const int sh = odd0 ^ ((d2 - P) & odd1 & 1) ^ (DIM == 3 ? (d3 - P) & odd12 & 1 : 0);
+          const double *st = ring + (size_t)slot * Gm::STAGE;
+          // rows whose (i_2 + delta_2, i_3 + delta_3) leaves the box have only
+          // zero coefficients in this group; skip when the whole warp is out
+          bool in23 = false;
+#pragma unroll
+          for (int r = 0; r < R; ++r) in23 = in23 || ((v2[r] >> d2) & (DIM == 3 ? v3[r] >> d3 : 1u) & 1u);
+          // the slot is free once the group's operands are in registers
+          auto release = [&]() {
+            __syncwarp();
+            if (lane == 0)
+              asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[slot])) : "memory");
+          };
+          if (!__any_sync(0xffffffffu, in23)) {
+            release();
+          } else {
+            // HALF: a mirrored run is read one row late when its start row was odd
+            if constexpr (R == 1) {
+              const double *cf = st + t0;
+              const double *xw = st + W * RS + t0 + sh;       // xw[j] = x[row + off - P + j]
+              double c[W], x[W];
+#pragma unroll
+              for (int j = 0; j < W; ++j) {
+                const int hs = HALF && ob + j < a.oc ? (int)((a.shH & 1) ^ sh ^ (j & 1)) : 0;
+                c[j] = cf[j * RS + hs];
+                x[j] = xw[j];
+              }
+              release();
+#pragma unroll
+              for (int j = 0; j < W; ++j) acc[0][j & 1] = fma(c[j], x[j], acc[0][j & 1]);
+            } else if constexpr (HALF) {
+              // rows row, row + 1: two 8-byte loads per run (no branch on the
+              // shift); x[row + off - P + j] = xv[j + sh], of the next row xv[j + 1 + sh]
+              const double *cf = st + t0;
+              const double2 *xb = reinterpret_cast<const double2 *>(st + W * RS + t0);
+              double xv[NV];
+#pragma unroll
+              for (int m = 0; m < NV / 2; ++m) { const double2 v = xb[m]; xv[2 * m] = v.x; xv[2 * m + 1] = v.y; }
+              double c0[W], c1[W];
+#pragma unroll
+              for (int j = 0; j < W; ++j) {
+                const int hs = ob + j < a.oc ? (int)((a.shH & 1) ^ sh ^ (j & 1)) : 0;
+                c0[j] = cf[j * RS + hs];
+                c1[j] = cf[j * RS + hs + 1];
+              }
+              release();
+#pragma unroll
+              for (int j = 0; j < W; ++j) {
+                const double xa = sh ? xv[j + 1] : xv[j], xc = sh ? xv[j + 2] : xv[j + 1];
+                acc[0][j & 1] = fma(c0[j], xa, acc[0][j & 1]);
+                acc[1][j & 1] = fma(c1[j], xc, acc[1][j & 1]);
+              }
+            } else {
+              // rows row, row + 1: coefficients c[j] = (S[o_j][row], S[o_j][row + 1]);
+              // x[row + off - P + j] = xv[j + sh], x[row + 1 + off - P + j] = xv[j + 1 + sh]
+              const double2 *cf = reinterpret_cast<const double2 *>(st + t0);
+              const double2 *xb = reinterpret_cast<const double2 *>(st + W * kTile + t0);
+              double xv[NV];
+#pragma unroll
+              for (int m = 0; m < NV / 2; ++m) { const double2 v = xb[m]; xv[2 * m] = v.x; xv[2 * m + 1] = v.y; }
+              if (sh == 0) {
+#pragma unroll
+                for (int j = 0; j < W; ++j) {
+                  const double2 c = cf[j * (kTile / 2)];
+                  acc[0][j & 1] = fma(c.x, xv[j], acc[0][j & 1]);
+                  acc[1][j & 1] = fma(c.y, xv[j + 1], acc[1][j & 1]);
+                }
+              } else {
+#pragma unroll
+                for (int j = 0; j < W; ++j) {
+                  const double2 c = cf[j * (kTile / 2)];
+                  acc[0][j & 1] = fma(c.x, xv[j + 1], acc[0][j & 1]);
+                  acc[1][j & 1] = fma(c.y, xv[j + 2], acc[1][j & 1]);
+                }
+              }
+              release();
+            }
+          }
+          if (++slot == kStages) { slot = 0; ++turn; }
+        }
+      }
+      if (!ok) break;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        if (!live[r]) continue;
+        const double ax = acc[r][0] + acc[r][1];
+        if (MODE == 0) {
+          a.y[row + r] = ax;
+          dot = fma(a.x[row + r], ax, dot);
         } else {
-          // rows row, row + 1: coefficients cf[j] = (S[o_j][row], S[o_j][row + 1]);
-          // x[row + off - P + j] = xv[j + sh], x[row + 1 + off - P + j] = xv[j + 1 + sh]
-          const double2 *cf = reinterpret_cast<const double2 *>(st + 2 * tid);
-          const double2 *xb = reinterpret_cast<const double2 *>(st + W * kTile + 2 * tid);
-          constexpr int NP = (W + 1) / 2;                  // pairs covering W + 1 values
-          double xv[2 * NP + 2];
-          if (sh == 0) {
-#pragma unroll
-            for (int m = 0; m < NP; ++m) { const double2 v = xb[m]; xv[2 * m] = v.x; xv[2 * m + 1] = v.y; }
-#pragma unroll
-            for (int j = 0; j < W; ++j) {
-              const double2 c = cf[j * (kTile / 2)];
-              acc[0] = fma(c.x, xv[j], acc[0]);
-              acc[1] = fma(c.y, xv[j + 1], acc[1]);
-            }
-          } else {
-#pragma unroll
-            for (int m = 0; m < NP + 1; ++m) { const double2 v = xb[m]; xv[2 * m] = v.x; xv[2 * m + 1] = v.y; }
-#pragma unroll
-            for (int j = 0; j < W; ++j) {
-              const double2 c = cf[j * (kTile / 2)];
-              acc[0] = fma(c.x, xv[j + 1], acc[0]);
-              acc[1] = fma(c.y, xv[j + 2], acc[1]);
-            }
-          }
-        }
-      }
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[slot])) : "memory");
-      if (g == G - 1) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          if (!live[r]) continue;
-          const double ax = acc[r];
-          if (MODE == 0) {
-            a.y[row + r] = ax;
-            dot = fma(a.x[row + r], ax, dot);
-          } else {
-            const double rr = a.b[row + r] - ax;
-            a.y[row + r] = rr;
-            dot = fma(rr, rr, dot);
-            if (a.z) dot2 = fma(rr, a.z[row + r], dot2);
-          }
+          const double rr = a.b[row + r] - ax;
+          a.y[row + r] = rr;
+          dot = fma(rr, rr, dot);
+          if (a.z) dot2 = fma(rr, a.z[row + r], dot2);
         }
       }
     }
@@ -441,6 +462,31 @@ igafd_status per_sm_of(Kern kern, int block, size_t smem, std::atomic<unsigned l
   }
   *out = per_sm[dev & 63].load();
   return IGAFD_OK;
+}
+
+// Rows per tile for N rows on `sms` SMs with `per_sm` resident CTAs each. The
+// CTAs of an SM share its FP64 pipe and every CTA walks its tiles in turn, so
+// the product takes as many rounds as the CTA with most tiles, each as long as
+// the rows in flight on an SM in a round (and some per round), or as one
+// tile's latency (measured at p = 3: 117 clocks per FMA of a chain with 2
+// warps on the SM, 139 with 7, where the pipe takes 16 per warp). With 256-row
+// tiles only, the last round of a mid-sized patch ran on few CTAs and a small
+// patch on few SMs: (61, 90, 47) at p = 4 took 373 us, now 319 (299 us of FP64
+// work); (20, 20, 20) at p = 3 took 35 us, now 24. Ties go to the larger tile.
+inline int tile_rows(long long N, int sms, int per_sm, int step) {
+  int best = kTile;
+  double cost = -1.0;
+  for (int h = kTile; h >= 64; h -= step) {
+    const long long tiles = (N + h - 1) / h, ctas = (long long)sms * per_sm;
+    const long long rounds = (tiles + ctas - 1) / ctas;
+    const double rows = (double)h * (rounds > 1 ? per_sm : (double)((tiles + sms - 1) / sms));
+    const double w = rows + 48.0 > 215.0 + 0.3 * rows ? rows + 48.0 : 215.0 + 0.3 * rows;
+    if (cost < 0.0 || rounds * w < cost) {
+      cost = rounds * w;
+      best = h;
+    }
+  }
+  return best;
 }
 
 }  // namespace
