@@ -15,7 +15,7 @@
 // with ea_m the largest exponent field of row m and eb_j that of row j of B
 // (U_k^T or U_k, split at set-up). Digits are exact in FP16; the FP32
 // accumulators of tcgen05.mma hold the leading groups' integers exactly (see
-// kStepTab). Groups g <= 5 are kept (21 digit products); their accumulators
+// Steps). Groups g <= 5 are kept (21 digit products); their accumulators
 // are summed as 64-bit integers and rounded to FP64 once. In units of 2^-53
 // of the result's norm, a product's error is 0.4-1.8 (0.4 unless one factor's
 // entries decay along the sum) where the FP64 FMA chain of the SIMT kernel
@@ -23,18 +23,19 @@
 // multiplies the integer result before that rounding. No FP64 instruction is
 // executed (each would issue at the 2-per-clock rate).
 //
-// Measured: 181 us per apply at n = 128 (SIMT: 3.10 ms), 103 us at
-// (95, 61, 77) (SIMT: 0.98 ms). A pass at n = 128 (about 25 us) is bound by
-// integer instructions (64 lanes per clock per SM): splitting the rows 4 us,
-// the MMAs with the summation of their accumulators 9 us (the MMAs alone 5),
-// rounding 5 us, the rest loads and the launch.
+// Measured: 170 us per apply at n = 128 (SIMT: 3.10 ms), 95 us at (95, 61, 77)
+// (SIMT: 0.98 ms). A pass at n = 128 is bound by integer instructions (64
+// lanes per clock per SM, conversions 16): 20 us, of which reading and
+// splitting the rows 6 us, the MMAs with the summation of their accumulators
+// 9 us (the MMAs alone 5), the last rounding 2.5 us; about 6 us pass between
+// two launches.
 //
 // A CTA takes 128 rows (the other directions' indices) and up to 128 columns.
 // A's digits live in tensor memory (6 slices of K/2 columns: 384 of 512 at
 // K = 128), where each thread writes the digits of its own row; B's digits
-// lie in shared memory (6 x 32 KB at n = 128); two accumulators of kNS columns
-// take the rest of tensor memory: one warp issues the products of a step into
-// one while the other warps read the previous one.
+// lie in shared memory (6 x 32 KB at n = 128); two accumulators of 64 columns
+// take the rest of tensor memory: the products of a step go into one while the
+// previous one is read.
 //
 // Directions are contracted in the order 3, 2, 1 and back 1, 3, 2: in four of
 // the six products (three of four in 2D) the row index is then contiguous in
@@ -53,12 +54,9 @@
 namespace {
 
 constexpr int kM = 128;                 // rows per CTA (MMA M, TMEM lanes)
-constexpr int kWorkers = 512;           // 4 warps per lane quarter; one more warp issues copies and MMAs
-constexpr int kThreads = kWorkers + 32;
+constexpr int kThreads = 512;           // 4 warps per lane quarter
+constexpr int kWarps = kThreads / 32;
 constexpr int kSlices = 6;              // digits per operand
-constexpr int kBits = 10;               // bits per digit
-constexpr int kNS = 64;                 // columns per accumulator
-constexpr int kFirst = 3;               // slices of B fetched before the input is read
 constexpr int kTrans = 16 * 32 * 17 * 8;// bytes of the transposition buffers
 constexpr long long kSpin = 1ll << 26;  // bounded waits
 // X + kBias = sum_s (digit_s + 512) 1024^(5-s): every 10-bit field is then the
@@ -72,7 +70,7 @@ struct SplitArgs {
   long long M;            // rows
   int F;                  // rows m = hi F + lo
   long long in_hi, in_lo, in_k, out_hi, out_lo, out_n;   // element strides
-  int K, Kp;              // contracted length, padded to a multiple of 32
+  int K, Kp;              // contracted length, padded to a multiple of 32 (the kernel's KP)
   int N, Np, NT;          // columns, padded to 16; columns per CTA (multiple of 16)
   const unsigned char *img;   // digits of B: [slice][64-wide K chunk][Np][128 B], swizzled
   const int *eb;              // exponent field of each row of B
@@ -88,10 +86,16 @@ struct SplitArgs {
 // |a| <= 2^9 and, over U_k's entries, |b| of half its 2^9 on average, so their
 // sums over 64 terms stay below 2^23 per product (2^22 with a_0). Group 3
 // weighs 2^-30 of group 0: a rounding there is below the result's last bit.
-struct Step { signed char g, c0, c1; };
-__constant__ Step kStepTab[2][8] = {
-    {{0, 0, 2}, {1, 0, 2}, {2, 0, 2}, {3, 0, 2}, {4, 0, 2}, {5, 0, 2}},
-    {{0, 0, 2}, {1, 0, 1}, {1, 1, 2}, {2, 0, 1}, {2, 1, 2}, {3, 0, 2}, {4, 0, 2}, {5, 0, 2}}};
+struct Step { int g, c0, c1; };
+template <int KP> struct Steps {
+  static constexpr int kCount = KP > 64 ? 8 : 6;
+  __host__ __device__ static constexpr Step at(int i) {
+    if (KP <= 64) return Step{i, 0, 1};
+    if (i == 0) return Step{0, 0, 2};
+    if (i < 5) return Step{(i + 1) / 2, (i - 1) % 2, (i - 1) % 2 + 1};
+    return Step{i - 2, 0, 2};
+  }
+};
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -218,33 +222,44 @@ __device__ __forceinline__ double round_fixed(long long T, int E, double lam, bo
                           zero ? 0 : (int)(uint32_t)q);
 }
 
-template <bool LAM>
-__global__ void __launch_bounds__(kThreads, 1) split_pass_kernel(SplitArgs a) {
+// Columns per accumulator and CTAs per SM: with K <= 64 two CTAs fit (256 TMEM
+// columns and half the shared memory each), so one's MMAs and the start of the
+// next launch overlap the other's integer work.
+constexpr int acc_cols(int KP) { return KP > 64 ? 64 : 32; }
+constexpr int ctas_per_sm(int KP) { return KP > 64 ? 1 : 2; }
+// slices of B fetched before the input is read (the rest of B's shared memory
+// holds the transposition buffers until then)
+constexpr int first_slices(int KP) { return KP > 64 ? 3 : 1; }
+template <int KP, bool LAM>
+__global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(SplitArgs a) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char *sB = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ uint64_t bar_b[2], bar_a[kSlices], bar_full[2], bar_empty[2];
+  __shared__ uint64_t bar_b[2], bar_full[2], bar_empty[2];
   __shared__ uint32_t tmem_slot;
   __shared__ unsigned short s_ea[4][kM], s_eb[kM];
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = (int)blockIdx.y * a.NT;
   const int NTc = a.Np - n0 < a.NT ? a.Np - n0 : a.NT;     // columns of this CTA
-  const int nkc = (a.Kp + 63) >> 6;
-  const int slice_bytes = nkc * a.NT * 128;
-  const int scols = a.Kp >> 1;                             // TMEM columns per slice of A
-  const int dbase = kSlices * scols;                       // accumulators: 2 x kNS columns
-  const int two = nkc > 1 ? 1 : 0;
-  const int per = two ? 8 : 6;                             // steps per column block
+  constexpr int nkc = (KP + 63) / 64;                      // 64-wide K chunks
+  constexpr int KS = KP / 16;                              // MMAs per digit product
+  constexpr int scols = KP / 2;                            // TMEM columns per slice of A
+  constexpr int dbase = kSlices * scols;                   // two accumulators follow
+  constexpr int per = Steps<KP>::kCount;                   // steps per column block
+  constexpr int kNS = acc_cols(KP), kFirst = first_slices(KP);
+  constexpr int kTmem = dbase + 2 * kNS > 256 ? 512 : 256; // allocated columns
+  // B in shared memory: [slice][chunk][128 rows][128 B] (row strides fixed, so
+  // that descriptors are constants apart from the column block)
+  constexpr int kChunk = kM * 128;
+  constexpr int slice_bytes = nkc * kChunk;
   const int nsub = (NTc + kNS - 1) / kNS;
-  const bool issuer = tid == kWorkers;                     // lane 0 of the last warp
 
-  if (issuer) {
+  if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bar_b[i], 1);
       mbar_init(&bar_full[i], 1);
-      mbar_init(&bar_empty[i], kWorkers / 32);
+      mbar_init(&bar_empty[i], kWarps);
     }
-    for (int i = 0; i < kSlices; ++i) mbar_init(&bar_a[i], kWorkers / 32);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_fail = 0;
   }
@@ -256,16 +271,17 @@ __global__ void __launch_bounds__(kThreads, 1) split_pass_kernel(SplitArgs a) {
       for (int c = 0; c < nkc; ++c)
         asm volatile(
             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                smem_u32(sB + (size_t)s * slice_bytes + (size_t)c * a.NT * 128)),
+                smem_u32(sB + (size_t)s * slice_bytes + (size_t)c * kChunk)),
             "l"(a.img + ((size_t)(s * nkc + c) * a.Np + n0) * 128), "r"((uint32_t)(NTc * 128)),
             "r"(smem_u32(bar))
             : "memory");
   };
-  if (warp == kWorkers / 32) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
-        smem_u32(&tmem_slot)));
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_slot)),
+                 "n"(kTmem));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    if (issuer) load_slices(0, kFirst, &bar_b[0]);
+    if (lane == 0) load_slices(0, kFirst, &bar_b[0]);
   }
   for (int n = tid; n < NTc; n += kThreads)
     s_eb[n] = (unsigned short)(n0 + n < a.N ? a.eb[n0 + n] : 1);
@@ -277,241 +293,246 @@ __global__ void __launch_bounds__(kThreads, 1) split_pass_kernel(SplitArgs a) {
   pdl_wait();
   pdl_trigger();
   if (a.done && *a.done != 0.0) {                          // uniform
-    if (issuer) wait_on(&bar_b[0], 0, &s_fail);
+    if (tid == 0) wait_on(&bar_b[0], 0, &s_fail);
     __syncthreads();
     if (warp == 0)
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmem));
     return;
   }
 
-  if (warp == kWorkers / 32) {
-    // ---- copies and MMAs: one elected lane issues (chosen by elect.sync, so
-    // that descriptors stay in uniform registers: an MMA then issues in 31
-    // clocks, its execution time, instead of 45-120 from a lane picked by its
-    // index) ----
-    __syncthreads();                                       // (the workers' exponent exchange)
+  // ---- A: this thread's row (lane 32 q + lane) and K range [kq KQ, kq KQ + KQ) ----
+  const int q = warp & 3, kq = warp >> 2;
+  constexpr int KQ = KP / 4;                             // 8, 16, 24 or 32
+  const int lrow = q * 32 + lane;
+  const long long m = (long long)blockIdx.x * kM + lrow;
+  const bool row_ok = m < a.M;
+  const long long hi = row_ok ? m / a.F : 0, lo = row_ok ? m - hi * a.F : 0;
+  const int k0 = kq * KQ;
+  const uint32_t lanes = (uint32_t)(q * 32) << 16;
+  int ea;
+  {
+    double x[KQ];
+    if (a.in_k != 1) {
+      const double *src = a.in + hi * a.in_hi + lo * a.in_lo + (long long)k0 * a.in_k;
+#pragma unroll
+      for (int i = 0; i < KQ; ++i)
+        x[i] = (row_ok && k0 + i < a.K) ? __ldg(src + (long long)i * a.in_k) : 0.0;
+    } else {
+      // rows contiguous in K: a warp reads runs of two rows at a time and
+      // transposes through its own buffer (in the part of shared memory that
+      // the later digits of B take afterwards)
+      constexpr int HP = (KQ + 15) / 16;                 // pieces of 16 elements
+      double *buf = reinterpret_cast<double *>(sB + (size_t)kFirst * slice_bytes) + warp * 32 * 17;
+      const long long base = row_ok ? hi * a.in_hi + lo * a.in_lo : -1;
+      const int cc = lane & 15;
+      double y[HP][16];
+#pragma unroll
+      for (int h = 0; h < HP; ++h) {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          const int k = k0 + 16 * h + cc;
+          const long long b = __shfl_sync(0xffffffffu, base, 2 * t + (lane >> 4));
+          const bool ok = b >= 0 && 16 * h + cc < KQ && k < a.K;
+          y[h][t] = ok ? __ldg(a.in + b + k) : 0.0;
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < HP; ++h) {
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < 16; ++t) buf[(2 * t + (lane >> 4)) * 17 + cc] = y[h][t];
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < 16; ++t)
+          if (16 * h + t < KQ) x[16 * h + t] = buf[lane * 17 + t];
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (LAM && row_ok && (lane & 15) == 0) {              // the divide's table, used last
+      const double *t = a.inv_lam + hi * a.out_hi + lo * a.out_lo + (long long)n0 * a.out_n;
+      for (int n = kq; n < NTc && n0 + n < a.N; n += 4)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(t + (long long)n * a.out_n));
+    }
+    int em = 1;
+#pragma unroll
+    for (int i = 0; i < KQ; ++i) em = max(em, exp_field((uint32_t)__double2hiint(x[i])));
+    s_ea[kq][lrow] = (unsigned short)em;
+    __syncthreads();
+    if (tid == 0) load_slices(kFirst, kSlices, &bar_b[1]);
+    ea = max(max((int)s_ea[0][lrow], (int)s_ea[1][lrow]), max((int)s_ea[2][lrow], (int)s_ea[3][lrow]));
+    uint32_t w1[KQ], w0[KQ];
+#pragma unroll
+    for (int i = 0; i < KQ; ++i) biased_fixed<58>(x[i], ea, w1[i], w0[i]);
+    auto put = [&](int s, auto pos, const uint32_t *w) {
+      constexpr int POS = decltype(pos)::value;
+#pragma unroll
+      for (int b = 0; b < KQ / 8; ++b)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                         tmem + lanes + (uint32_t)(s * scols + (k0 >> 1) + 4 * b)),
+                     "r"(digit2<POS>(w[8 * b], w[8 * b + 1])),
+                     "r"(digit2<POS>(w[8 * b + 2], w[8 * b + 3])),
+                     "r"(digit2<POS>(w[8 * b + 4], w[8 * b + 5])),
+                     "r"(digit2<POS>(w[8 * b + 6], w[8 * b + 7]))
+                     : "memory");
+    };
+    put(0, std::integral_constant<int, 2>{}, w1);
+    put(1, std::integral_constant<int, 1>{}, w1);
+    put(2, std::integral_constant<int, 0>{}, w1);
+    put(3, std::integral_constant<int, 2>{}, w0);
+    put(4, std::integral_constant<int, 1>{}, w0);
+    put(5, std::integral_constant<int, 0>{}, w0);
+  }
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+
+  // ---- digit products. A step's MMAs are issued by one elected lane of warp
+  // step mod 16, while the others sum the step before. (Elected by elect.sync,
+  // so that descriptors stay in uniform registers: an MMA then issues in its
+  // execution time, 31 clocks, instead of 45-120 from a lane picked by index;
+  // a seventeenth warp for the issue alone would leave 96 registers a thread
+  // and spill.) ----
+  const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+  const uint64_t b0 = sw128_desc(smem_u32(sB));
+  bool ok = true;
+  auto issue = [&](auto step, int sub, int st) {           // one warp
+    constexpr int i = decltype(step)::value;
+    constexpr Step p = Steps<KP>::at(i);
+    const int buf = st & 1;
+    if (i == 0 && sub == 0) ok = ok && wait_on(&bar_b[0], 0, &s_fail);
+    if (p.g >= kFirst && sub == 0) ok = ok && wait_on(&bar_b[1], 0, &s_fail);
+    if (st >= 2) ok = ok && wait_on(&bar_empty[buf], (uint32_t)(((st >> 1) - 1) & 1), &s_fail);
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) return;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const int nc = NTc - sub * kNS < kNS ? NTc - sub * kNS : kNS;
+    const uint32_t idesc = (1u << 4) | ((uint32_t)(nc >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
+    const uint32_t d = tm + (uint32_t)(dbase + buf * kNS);
     uint32_t elected;
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
                  : "=r"(elected));
-    if (issuer) load_slices(kFirst, kSlices, &bar_b[1]);
-    __syncwarp();
-    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-    const uint32_t cstep = (uint32_t)(a.NT * 128) >> 4;    // descriptor steps (16 bytes)
-    const uint64_t b0 = sw128_desc(smem_u32(sB));
-    const int ksteps = a.Kp >> 4;
-    int st = 0, slices = 0;                                // slices of A known to be ready
-    bool ok = wait_on(&bar_b[0], 0, &s_fail);
-    for (int sub = 0; ok && sub < nsub; ++sub) {
-      const int nc = NTc - sub * kNS < kNS ? NTc - sub * kNS : kNS;
-      const uint32_t idesc = (1u << 4) | ((uint32_t)(nc >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
-      for (int i = 0; ok && i < per; ++i, ++st) {
-        const Step p = kStepTab[two][i];
-        if (sub == 0) {
-          for (; ok && slices <= p.g; ++slices) {
-            ok = wait_on(&bar_a[slices], 0, &s_fail);
-            if (ok && slices == kFirst) ok = wait_on(&bar_b[1], 0, &s_fail);
-          }
-        }
-        const int buf = st & 1;
-        if (ok && st >= 2) ok = wait_on(&bar_empty[buf], (uint32_t)(((st >> 1) - 1) & 1), &s_fail);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tm + (uint32_t)(dbase + buf * kNS);
-        if (elected) {
-          uint32_t acc = 0u;
-          for (int s = 0; s <= p.g; ++s) {
-            for (int c = p.c0; c < p.c1 && c < nkc; ++c) {
-              const uint64_t bs = b0 + (uint32_t)(((p.g - s) * slice_bytes + sub * kNS * 128) >> 4) + c * cstep;
-              const uint32_t as = tm + (uint32_t)(s * scols + c * 32);
-              const int kn = ksteps - 4 * c;
+    const uint64_t bsub = b0 + (uint32_t)(sub * kNS * 128 >> 4);   // (descriptor steps of 16 bytes)
+    if (elected) {
 #pragma unroll
-              for (int ks = 0; ks < 4; ++ks) {
-                if (ks < kn)
-                  asm volatile(
-                      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
-                      "r"(as + (uint32_t)(ks * 8)), "l"(bs + (uint64_t)(ks * 2)), "r"(idesc), "r"(acc));
-                acc = 1u;
-              }
-            }
-          }
+      for (int sl = 0; sl <= p.g; ++sl) {
+        const uint64_t bs = bsub + (uint32_t)((p.g - sl) * slice_bytes >> 4);
+#pragma unroll
+        for (int ks = 4 * p.c0; ks < KS && ks < 4 * p.c1; ++ks) {
+          const uint32_t acc = sl == 0 && ks == 4 * p.c0 ? 0u : 1u;
           asm volatile(
-              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                  smem_u32(&bar_full[buf]))
-              : "memory");
+              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+              " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+              "r"(tm + (uint32_t)(sl * scols + ks * 8)),
+              "l"(bs + (uint64_t)((ks >> 2) * (kChunk >> 4) + (ks & 3) * 2)), "r"(idesc), "r"(acc));
         }
-        __syncwarp();
       }
+      asm volatile(
+          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+              smem_u32(&bar_full[buf]))
+          : "memory");
     }
-    if (!ok) s_fail = 1;
-    // the copies this warp issued land before shared memory is released
-    wait_on(&bar_b[0], 0, &s_fail);
-    wait_on(&bar_b[1], 0, &s_fail);
-  } else {
-    // ---- A: this thread's row (lane 32 q + lane) and K range [kq KQ, kq KQ + KQ) ----
-    const int q = warp & 3, kq = warp >> 2;
-    const int KQ = a.Kp >> 2;                              // 8, 16, 24 or 32
-    const int lrow = q * 32 + lane;
-    const long long m = (long long)blockIdx.x * kM + lrow;
-    const bool row_ok = m < a.M;
-    const long long hi = row_ok ? m / a.F : 0, lo = row_ok ? m - hi * a.F : 0;
-    const int k0 = kq * KQ;
-    const uint32_t lanes = (uint32_t)(q * 32) << 16;
-    int ea;
-    {
-      double x[32];
-      if (a.in_k != 1) {
-        const double *src = a.in + hi * a.in_hi + lo * a.in_lo + (long long)k0 * a.in_k;
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          x[i] = (i < KQ && row_ok && k0 + i < a.K) ? __ldg(src + (long long)i * a.in_k) : 0.0;
-      } else {
-        // rows contiguous in K: a warp reads 128-byte runs of two rows at a
-        // time and transposes through its own buffer (in the part of shared
-        // memory that the later digits of B take afterwards)
-        double *buf = reinterpret_cast<double *>(sB + (size_t)kFirst * slice_bytes) + warp * 32 * 17;
-        const long long base = row_ok ? hi * a.in_hi + lo * a.in_lo : -1;
-        const int cc = lane & 15;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-#pragma unroll
-          for (int t = 0; t < 16; ++t) {
-            const int k = k0 + 16 * h + cc;
-            const long long b = __shfl_sync(0xffffffffu, base, 2 * t + (lane >> 4));
-            const bool ok = b >= 0 && 16 * h + cc < KQ && k < a.K;
-            x[16 * h + t] = ok ? __ldg(a.in + b + k) : 0.0;
-          }
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          __syncwarp();
-#pragma unroll
-          for (int t = 0; t < 16; ++t) buf[(2 * t + (lane >> 4)) * 17 + cc] = x[16 * h + t];
-          __syncwarp();
-#pragma unroll
-          for (int t = 0; t < 16; ++t) x[16 * h + t] = buf[lane * 17 + t];
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+  };
+  if (warp == 0) issue(std::integral_constant<int, 0>{}, 0, 0);
+  // ---- accumulators to integers, rounded once ----
+  constexpr int C = kNS / 4;                               // columns per thread in a block
+  const bool bad_row = ea == 0x7ff;
+  const long long ob = hi * a.out_hi + lo * a.out_lo;
+  int st = 0;
+  for (int sub = 0; sub < nsub; ++sub) {
+    long long T[C];
+    auto sum = [&](auto step) {
+      constexpr int i = decltype(step)::value;
+      constexpr int g = Steps<KP>::at(i).g;
+      const int buf = st & 1;
+      if (warp == ((st + 1) & (kWarps - 1)) && (i + 1 < per || sub + 1 < nsub))
+        issue(std::integral_constant<int, (i + 1) % per>{}, i + 1 < per ? sub : sub + 1, st + 1);
+      ok = ok && wait_on(&bar_full[buf], (uint32_t)((st >> 1) & 1), &s_fail);
+      ok = __all_sync(0xffffffffu, ok);
+      ++st;
+      if (!ok) {
+        s_fail = 1;
+        return;
       }
-      if (LAM && row_ok && (lane & 15) == 0) {              // the divide's table, used last
-        const double *t = a.inv_lam + hi * a.out_hi + lo * a.out_lo + (long long)n0 * a.out_n;
-        for (int n = kq; n < NTc && n0 + n < a.N; n += 4)
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(t + (long long)n * a.out_n));
-      }
-      int em = 1;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) em = max(em, exp_field((uint32_t)__double2hiint(x[i])));
-      s_ea[kq][lrow] = (unsigned short)em;
-      __syncthreads();
-      ea = max(max((int)s_ea[0][lrow], (int)s_ea[1][lrow]), max((int)s_ea[2][lrow], (int)s_ea[3][lrow]));
-      uint32_t w1[32], w0[32];
-#pragma unroll
-      for (int i = 0; i < 32; ++i)
-        if (i < KQ) biased_fixed<58>(x[i], ea, w1[i], w0[i]);
-      auto put = [&](int s, auto pos, const uint32_t *w) {
-        constexpr int POS = decltype(pos)::value;
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-          if (8 * b < KQ)
-            asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                             tmem + lanes + (uint32_t)(s * scols + (k0 >> 1) + 4 * b)),
-                         "r"(digit2<POS>(w[8 * b], w[8 * b + 1])),
-                         "r"(digit2<POS>(w[8 * b + 2], w[8 * b + 3])),
-                         "r"(digit2<POS>(w[8 * b + 4], w[8 * b + 5])),
-                         "r"(digit2<POS>(w[8 * b + 6], w[8 * b + 7]))
-                         : "memory");
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bar_a[s]);
-      };
-      put(0, std::integral_constant<int, 2>{}, w1);
-      put(1, std::integral_constant<int, 1>{}, w1);
-      put(2, std::integral_constant<int, 0>{}, w1);
-      put(3, std::integral_constant<int, 2>{}, w0);
-      put(4, std::integral_constant<int, 1>{}, w0);
-      put(5, std::integral_constant<int, 0>{}, w0);
-    }
-    // ---- accumulators to integers, rounded once ----
-    constexpr int C = kNS / 4;                             // columns per thread in a block
-    const bool bad_row = ea == 0x7ff;
-    const long long ob = hi * a.out_hi + lo * a.out_lo;
-    int st = 0;
-    bool ok = true;
-    for (int sub = 0; ok && sub < nsub; ++sub) {
-      long long T[C];
-      for (int i = 0; i < per; ++i, ++st) {
-        const int g = kStepTab[two][i].g, buf = st & 1;
-        ok = wait_on(&bar_full[buf], (uint32_t)((st >> 1) & 1), &s_fail);
-        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        uint32_t v[C];
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      uint32_t v[C];
+      const uint32_t dv = tmem + lanes + (uint32_t)(dbase + buf * kNS + kq * C);
+      if constexpr (C == 8)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
+                       "=r"(v[6]), "=r"(v[7])
+                     : "r"(dv));
+      else
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
             "%14,%15}, [%16];"
             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-              "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(tmem + lanes + (uint32_t)(dbase + buf * kNS + kq * C)));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bar_empty[buf]);
-        // T in units of 2^12 of group 5: |G_0| 2^38 <= 2^62; what is dropped
-        // of groups 4 and 5 is of the order of the groups not computed
-        if (g < 4) {
-          const int wt = 1 << (28 - 10 * (g > 0 ? g - 1 : 0));
-#pragma unroll
-          for (int c = 0; c < C; ++c) {
-            const int G = __float2int_rn(__uint_as_float(v[c]));
-            T[c] = g == 0 ? (long long)G << 38 : T[c] + (long long)G * wt;
-          }
-        } else {
-          const int rs = g == 4 ? 2 : 12, half = 1 << (rs - 1);
-#pragma unroll
-          for (int c = 0; c < C; ++c)
-            T[c] += (long long)((__float2int_rn(__uint_as_float(v[c])) + half) >> rs);
-        }
-      }
-      if (!ok || !row_ok) continue;
-      const int nl0 = sub * kNS + kq * C;                  // this thread's first column, and how many
-      const int ncol = min(C, min(NTc - nl0, a.N - n0 - nl0));
-      const long long o0 = ob + (long long)(n0 + nl0) * a.out_n;
-      double lam[C];
-#pragma unroll
-      for (int c = 0; c < C; ++c) lam[c] = LAM && c < ncol ? __ldg(a.inv_lam + o0 + c * a.out_n) : 1.0;
-      bool slow = bad_row;
+              "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+              "=r"(v[14]), "=r"(v[15])
+            : "r"(dv));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar_empty[buf]);
+      // T in units of 2^12 of group 5: |G_0| 2^38 <= 2^62; what is dropped of
+      // groups 4 and 5 is of the order of the groups not computed
 #pragma unroll
       for (int c = 0; c < C; ++c) {
-        const double y = round_fixed<LAM>(T[c], ea + (int)s_eb[(nl0 + c) & (kM - 1)] - 2099, lam[c], slow);
-        if (c < ncol) a.out[o0 + c * a.out_n] = y;
+        const int G = __float2int_rn(__uint_as_float(v[c]));
+        if (g == 0) T[c] = (long long)G << 38;
+        else if (g < 4) T[c] += (long long)G * (1 << (g > 0 && g < 4 ? 38 - 10 * g : 0));
+        else T[c] += (long long)(g == 4 ? (G + 2) >> 2 : (G + 2048) >> 12);
       }
-      if (slow) {                                          // rare: again, one by one
-#pragma unroll
-        for (int c = 0; c < C; ++c)
-          if (c < ncol)
-            a.out[o0 + c * a.out_n] =
-                bad_row ? __longlong_as_double(0x7ff8000000000000ll)
-                        : round_slow(T[c], ea + (int)s_eb[nl0 + c] - 2099, lam[c]);
-      }
+    };
+    sum(std::integral_constant<int, 0>{});
+    sum(std::integral_constant<int, 1>{});
+    sum(std::integral_constant<int, 2>{});
+    sum(std::integral_constant<int, 3>{});
+    sum(std::integral_constant<int, 4>{});
+    sum(std::integral_constant<int, 5>{});
+    if constexpr (per == 8) {
+      sum(std::integral_constant<int, 6>{});
+      sum(std::integral_constant<int, 7>{});
     }
-    if (!ok) s_fail = 1;
+    if (!ok || !row_ok) continue;
+    const int nl0 = sub * kNS + kq * C;                  // this thread's first column, and how many
+    const int ncol = min(C, min(NTc - nl0, a.N - n0 - nl0));
+    const long long o0 = ob + (long long)(n0 + nl0) * a.out_n;
+    double lam[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) lam[c] = LAM && c < ncol ? __ldg(a.inv_lam + o0 + c * a.out_n) : 1.0;
+    bool slow = bad_row;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      const double y = round_fixed<LAM>(T[c], ea + (int)s_eb[(nl0 + c) & (kM - 1)] - 2099, lam[c], slow);
+      if (c < ncol) a.out[o0 + c * a.out_n] = y;
+    }
+    if (slow) {                                          // rare: again, one by one
+#pragma unroll
+      for (int c = 0; c < C; ++c)
+        if (c < ncol)
+          a.out[o0 + c * a.out_n] =
+              bad_row ? __longlong_as_double(0x7ff8000000000000ll)
+                      : round_slow(T[c], ea + (int)s_eb[nl0 + c] - 2099, lam[c]);
+    }
   }
+  if (!ok) s_fail = 1;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (issuer && s_fail) {
+  if (tid == 0 && s_fail) {
     atomicExch(a.err, (int)IGAFD_ERR_TIMEOUT);
-    // a wait ran out: give the MMAs in flight a bounded chance to finish
-    // before TMEM is released
+    // a wait ran out: give the copies and MMAs in flight a bounded chance to
+    // finish before shared memory and TMEM are released
     const int none = 0;
+    wait_on(&bar_b[0], 0, &none);
+    wait_on(&bar_b[1], 0, &none);
     for (int i = 0; i < 2; ++i) {
       wait_on(&bar_full[i], 0, &none);
       wait_on(&bar_full[i], 1, &none);
     }
   }
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmem));
 }
 
 // Digits of B = U_k^T (transpose) or U_k as the shared-memory images of the
@@ -556,9 +577,9 @@ __global__ void __launch_bounds__(128) split_image_kernel(ImgBatch b) {
 
 int pad(int n, int to) { return (n + to - 1) / to * to; }
 
-size_t pass_smem(int Kp, int NT) {
-  const size_t slice = (size_t)((Kp + 63) / 64) * NT * 128;
-  const size_t a = kSlices * slice, b = kFirst * slice + kTrans;
+size_t pass_smem(int Kp) {
+  const size_t slice = (size_t)((Kp + 63) / 64) * kM * 128;
+  const size_t a = kSlices * slice, b = first_slices(Kp) * slice + kTrans;
   return 1024 + (a > b ? a : b);
 }
 
@@ -634,17 +655,22 @@ static igafd_status launch_pass(igafd_patch *P, int k, int dir, SplitArgs a, cud
   while (parts < 8 && tiles * parts * 2 <= P->num_sms && pad(a.Np, 32 * parts) / parts > 16) parts *= 2;
   a.NT = pad((a.Np + parts - 1) / parts, 16);
   parts = (a.Np + a.NT - 1) / a.NT;
-  const size_t smem = pass_smem(a.Kp, a.NT);
+  const size_t smem = pass_smem(a.Kp);
+  using Kern = void (*)(SplitArgs);
+  static const Kern kerns[4][2] = {{split_pass_kernel<32, false>, split_pass_kernel<32, true>},
+                                   {split_pass_kernel<64, false>, split_pass_kernel<64, true>},
+                                   {split_pass_kernel<96, false>, split_pass_kernel<96, true>},
+                                   {split_pass_kernel<128, false>, split_pass_kernel<128, true>}};
   static std::atomic<unsigned long long> attr_set{0};
   const unsigned long long bit = 1ull << (P->dev & 63);
   if (!(attr_set.load() & bit)) {
-    for (auto kern : {split_pass_kernel<false>, split_pass_kernel<true>})
-      IGAFD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)pass_smem(128, 128)));
+    for (int i = 0; i < 8; ++i)
+      IGAFD_CUDA(cudaFuncSetAttribute(kerns[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)pass_smem(128)));
     attr_set.fetch_or(bit);
   }
-  IGAFD_CUDA(igafd_launch(a.inv_lam ? split_pass_kernel<true> : split_pass_kernel<false>,
-                          dim3((unsigned)tiles, (unsigned)parts), dim3(kThreads), smem, s, a));
+  IGAFD_CUDA(igafd_launch(kerns[a.Kp / 32 - 1][a.inv_lam ? 1 : 0], dim3((unsigned)tiles, (unsigned)parts),
+                          dim3(kThreads), smem, s, a));
   IGAFD_LAUNCHED(1);
   return IGAFD_OK;
 }
