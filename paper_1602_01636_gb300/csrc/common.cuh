@@ -135,7 +135,7 @@ struct igafd_patch {
   int fd_tile[3][4];            // per operand type: per-mode kernel's rows per CTA (64 or 128; 0 =
                                 // 128), column split (2 = two column tiles, else one), K stages (3,
                                 // else 2); pencil kernel's columns per CTA (64 or 128; 0 = 128)
-  int eig_route;                // 0: FP32 Jacobi + FP64 refinement where n_k <= 128; 1: FP64 Jacobi
+  int eig_route;                // 0: FP32 start + FP64 refinement; 1: FP64 Jacobi
   int eig_used[3];              // route each direction took: 0 refined, 1 FP64 Jacobi
   double eig_check[3][2];       // refined route's final check (orthogonality, off-diagonal)
   double *eig_work;             // eigen-setup scratch (kept for re-setups)

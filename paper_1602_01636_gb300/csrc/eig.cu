@@ -8,8 +8,8 @@
 //   positive.
 //
 // Two routes:
-//   fast (n <= 128): an FP32 start in one CTA per pencil, all in shared
-//     memory -- banded Cholesky M = L L^T, K~ = L^{-1} K L^{-T}, Householder
+//   fast: an FP32 start in one CTA per pencil (n <= 128: all in shared memory;
+//     above: from L1 and L2) -- banded Cholesky M = L L^T, K~ = L^{-1} K L^{-T}, Householder
 //     tridiagonalisation T = Q^T K~ Q, every eigenvalue of T by bisection on
 //     Sturm counts, eigenvectors of T by inverse iteration (2 steps; members of
 //     a cluster of eigenvalues closer than 1e-5 ||T|| are solved in turn and
@@ -28,7 +28,7 @@
 //     reductions use one warp per row (GB300's FP64 rate per SM is low). The
 //     result is checked (max |X^T M X - I| and max |offdiag S| / max |diag S|
 //     <= 1e-12); a pencil that fails takes the other route.
-//   FP64 (n > 128, or fallback): banded Cholesky and K~ in FP64, cyclic
+//   FP64 (fallback, or on request): banded Cholesky and K~ in FP64, cyclic
 //     two-sided Jacobi with a round-robin (tournament) ordering, n/2 disjoint
 //     rotations in parallel, U = L^{-T} U~.
 // Directions with the same knot vector have the same pencils; their
@@ -246,6 +246,7 @@ __global__ void __launch_bounds__(1024) tri32_kernel(EigJob *jobs, int allow_fas
   if (tid == 0)
     for (int i = 1; i < kScal; ++i) jb.sc[i] = 0.0;   // also zeroes state, counter, maxima
   if (!allow_fast || n > kFastMaxN || p >= kMaxBand) {
+    // the FP64 route, unless big32_kernel takes the pencil next
     if (tid == 0) *jb.state = 1;
     return;
   }
@@ -614,6 +615,363 @@ __global__ void __launch_bounds__(1024) tri32_kernel(EigJob *jobs, int allow_fas
   if (tid == 0) *jb.state = 0;
 }
 
+// ---- fast route, step 1 for n > kFastMaxN: the same start from L2 ----
+// The matrices do not fit in shared memory: K~ and the reflectors (row k holds
+// reflector k) live in the first half of jb.A, the eigenvectors of T in the
+// second, the pivot rows of the inverse iteration in jb.V (all solves at
+// once). Every pass over a matrix walks its rows, coalesced; L1 holds much of
+// it up to n of about 200. One CTA does the start up to T's eigenvectors;
+// back32_kernel takes them back to the pencil's, columns spread over CTAs.
+// Measured, the whole eigendecomposition with the refinement: 1.5 ms at n =
+// 150, 2.1 at 192, 6 at 300, 24 at 512, where FP64 Jacobi took 73, 161, 647 and
+// 3600 ms. Bound by the tridiagonalisation's passes over the matrix (one CTA).
+constexpr int kBigMaxN = 1024;
+
+// eight threads per eigenvalue: 9-way multisection on Sturm counts (the
+// interval shrinks by 9 per round)
+__device__ __forceinline__ float multisect(const float *dd, const float *e2, int n, int ev, float lo,
+                                           float hi, float pivmin, int lane) {
+  const int sub = lane & 7, base = lane & ~7;
+  for (int it = 0; it < 9; ++it) {
+    const float x = lo + (hi - lo) * (float)(sub + 1) * (1.0f / 9.0f);
+    int cnt = 0;
+    float q = dd[0] - x;
+    for (int j = 0;; ++j) {
+      if (fabsf(q) < pivmin) q = -pivmin;
+      cnt += q < 0.0f;
+      if (j == n - 1) break;
+      q = (dd[j + 1] - x) - __fdividef(e2[j], q);
+    }
+    // bit s of grp: point s has at most ev eigenvalues below it; the
+    // eigenvalue lies between the highest such point and the next one
+    const unsigned grp = (__ballot_sync(0xffffffffu, cnt <= ev) >> base) & 0xffu;
+    const int s_lo = grp ? 31 - __clz(grp) : -1;
+    const float xlo = __shfl_sync(0xffffffffu, x, base + (s_lo >= 0 ? s_lo : 0));
+    const float xhi = __shfl_sync(0xffffffffu, x, base + (s_lo + 1 <= 7 ? s_lo + 1 : 7));
+    if (s_lo >= 0) lo = xlo;
+    if (s_lo < 7) hi = xhi;
+  }
+  return 0.5f * (lo + hi);
+}
+
+// banded Cholesky M = L L^T in FP32 by one warp (Lb[i * kMaxBand + d] =
+// L[i][i - d], rdg = 1 / l_ii); false when M is not positive definite
+__device__ __forceinline__ bool band_cholesky32(float *Lb, float *rdg, int n, int p, int lane) {
+  int fail = 0;
+  for (int k = 0; k < n; ++k) {
+    const float dk = Lb[k * kMaxBand];
+    __syncwarp();
+    if (!(dk > 0.0f)) fail = 1;
+    const float r = dk > 0.0f ? rsqrtf(dk) : 1.0f;
+    const float lkk = dk > 0.0f ? dk * r : 1.0f;
+    if (lane == 0) { Lb[k * kMaxBand] = lkk; rdg[k] = r; }
+    if (lane >= 1 && lane <= p && k + lane < n) Lb[(k + lane) * kMaxBand + lane] *= r;
+    __syncwarp();
+    // L[k+a][k+b] -= L[k+a][k] L[k+b][k] for 1 <= b <= a <= p
+    for (int t = lane; t < p * p; t += 32) {
+      const int a = t / p + 1, b = t % p + 1;
+      if (b <= a && k + a < n)
+        Lb[(k + a) * kMaxBand + (a - b)] -= Lb[(k + a) * kMaxBand + a] * Lb[(k + b) * kMaxBand + b];
+    }
+    __syncwarp();
+  }
+  return !__any_sync(0xffffffffu, fail);
+}
+
+// shared memory (floats): seven vectors, 1 / l_ii and the band of L
+__host__ __device__ constexpr size_t big32_smem_floats(int n) { return (size_t)n * (8 + kMaxBand); }
+
+__global__ void __launch_bounds__(1024) big32_kernel(EigJob *jobs, int allow_fast) {
+  EigJob jb = jobs[blockIdx.x];
+  const int n = jb.n, p = jb.p;
+  if (!allow_fast || n <= kFastMaxN || p >= kMaxBand) return;   // tri32_kernel's pencils
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt / 32;
+  extern __shared__ float t32[];
+  float *vv = t32, *pw = vv + n, *dd = pw + n, *ee = dd + n, *e2 = ee + n, *bet = e2 + n, *lam = bet + n;
+  float *rdg = lam + n, *Lb = rdg + n;
+  __shared__ float s_f[4], s_nrm[32];
+  __shared__ int s_ok, s_start[kBigMaxN];
+  float *As = reinterpret_cast<float *>(jb.A), *Zs = As + (size_t)n * n;
+  float *P0 = reinterpret_cast<float *>(jb.V), *P1 = P0 + (size_t)n * n;
+  const size_t ld = n;
+  for (int t = tid; t < n * n; t += nt) As[t] = (float)jb.K[t];
+  for (int t = tid; t < n * kMaxBand; t += nt) {
+    const int i = t / kMaxBand, d = t % kMaxBand;
+    Lb[t] = (d <= p && i - d >= 0) ? (float)jb.M[(size_t)i * n + i - d] : 0.0f;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const bool ok = band_cholesky32(Lb, rdg, n, p, lane);
+    if (lane == 0) s_ok = ok;
+  }
+  __syncthreads();
+  if (!s_ok) {
+    if (tid == 0) *jb.state = 1;
+    return;
+  }
+  // K~ = L^{-1} K L^{-T}: columns of X = L^{-1} K by forward substitution,
+  // then those of L^{-1} X^T (= K~, symmetric)
+  auto forward = [&](float *B) {
+    for (int c = tid; c < n; c += nt) {
+      float w[kMaxBand - 1];
+#pragma unroll
+      for (int d = 0; d < kMaxBand - 1; ++d) w[d] = 0.0f;
+      for (int i = 0; i < n; ++i) {
+        float acc = B[i * ld + c];
+#pragma unroll
+        for (int d = 0; d < kMaxBand - 1; ++d)
+          if (d < p) acc -= Lb[i * kMaxBand + 1 + d] * w[d];
+        const float x = acc * rdg[i];
+        B[i * ld + c] = x;
+#pragma unroll
+        for (int d = kMaxBand - 2; d > 0; --d) w[d] = w[d - 1];
+        w[0] = x;
+      }
+    }
+    __syncthreads();
+  };
+  forward(As);
+  for (int t = tid; t < n * n; t += nt) Zs[(t % n) * ld + t / n] = As[t];
+  __syncthreads();
+  forward(Zs);
+  for (int t = tid; t < n * n; t += nt) {
+    const int i = t / n, j = t % n;
+    As[t] = 0.5f * (Zs[i * ld + j] + Zs[j * ld + i]);
+  }
+  __syncthreads();
+  {
+    // infinity norm of K~ (bounds its 2-norm): one warp per row
+    float mx = 0.0f;
+    for (int i = warp; i < n; i += nw) {
+      float rs = 0.0f;
+      for (int j = lane; j < n; j += 32) rs += fabsf(As[i * ld + j]);
+      mx = fmaxf(mx, warp_sum_f(rs));
+    }
+    if (lane == 0) s_nrm[warp] = mx;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    float m = 0.0f;
+    for (int w = 0; w < nw; ++w) m = fmaxf(m, s_nrm[w]);
+    jb.sc[0] = (double)m;
+  }
+  // Householder tridiagonalisation: step k zeroes A[k][k+2..]; reflector k
+  // stays in row k from column k + 1
+  for (int k = 0; k < n - 2; ++k) {
+    const int m = n - k - 1;
+    float *rowk = As + k * ld + k + 1;
+    if (warp == 0) {
+      float x2 = 0.0f, t2 = 0.0f;
+      for (int i = lane; i < m; i += 32) {
+        const float x = rowk[i];
+        x2 += x * x;
+        if (i > 0) { t2 += x * x; vv[i] = x; }
+      }
+      x2 = warp_sum_f(x2);
+      t2 = warp_sum_f(t2);
+      if (lane == 0) {
+        const float x0 = rowk[0];
+        float beta = 0.0f, alpha = x0;
+        if (t2 > 0.0f) {
+          const float nx = sqrtf(x2);
+          alpha = x0 >= 0.0f ? -nx : nx;
+          const float v0 = x0 - alpha;
+          beta = 2.0f / (t2 + v0 * v0);
+          vv[0] = v0;
+        }
+        s_f[0] = beta;
+        dd[k] = As[k * ld + k];
+        ee[k] = alpha;
+        bet[k] = beta;
+      }
+    }
+    __syncthreads();
+    const float beta = s_f[0];
+    if (beta == 0.0f) {                   // already tridiagonal in this row (uniform)
+      __syncthreads();
+      continue;
+    }
+    for (int r = warp; r < m; r += nw) {  // p = beta A_sub v
+      const float *row = As + (k + 1 + r) * ld + k + 1;
+      float acc = 0.0f;
+      for (int j = lane; j < m; j += 32) acc += row[j] * vv[j];
+      acc = warp_sum_f(acc);
+      if (lane == 0) pw[r] = beta * acc;
+    }
+    __syncthreads();
+    // K = beta/2 v.p (every warp computes it), w = p - K v, A_sub -= v w^T + w v^T
+    float vp = 0.0f;
+    for (int i = lane; i < m; i += 32) vp += vv[i] * pw[i];
+    const float K = 0.5f * beta * warp_sum_f(vp);
+    for (int i = warp; i < m; i += nw) {
+      const float vi = vv[i], wi = pw[i] - K * vi;
+      float *row = As + (k + 1 + i) * ld + k + 1;
+      for (int j = lane; j < m; j += 32) row[j] -= vi * (pw[j] - K * vv[j]) + wi * vv[j];
+    }
+    for (int i = tid; i < m; i += nt) rowk[i] = vv[i];
+    __syncthreads();
+  }
+  if (tid == 0) {
+    dd[n - 2] = As[(n - 2) * ld + n - 2];
+    ee[n - 2] = As[(n - 2) * ld + n - 1];
+    dd[n - 1] = As[(n - 1) * ld + n - 1];
+    bet[n - 2] = bet[n - 1] = 0.0f;
+  }
+  __syncthreads();
+  if (warp == 0) {                        // Gershgorin interval of T
+    float lo = 3.0e38f, hi = -3.0e38f, me2 = 0.0f;
+    for (int i = lane; i < n; i += 32) {
+      const float el = i > 0 ? fabsf(ee[i - 1]) : 0.0f, er = i < n - 1 ? fabsf(ee[i]) : 0.0f;
+      lo = fminf(lo, dd[i] - el - er);
+      hi = fmaxf(hi, dd[i] + el + er);
+      if (i < n - 1) { e2[i] = ee[i] * ee[i]; me2 = fmaxf(me2, e2[i]); }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      me2 = fmaxf(me2, __shfl_xor_sync(0xffffffffu, me2, o));
+    }
+    if (lane == 0) {
+      s_f[0] = lo; s_f[1] = hi;
+      s_f[2] = fmaxf(fabsf(lo), fabsf(hi));
+      s_f[3] = 1.0e-30f * fmaxf(1.0f, me2);      // smallest pivot of a Sturm sequence
+    }
+  }
+  __syncthreads();
+  const float tn = s_f[2];
+  for (int e0 = 0; e0 < n; e0 += nt / 8) {
+    const int ev = e0 + (tid >> 3);
+    const float l = multisect(dd, e2, n, min(ev, n - 1), s_f[0], s_f[1], s_f[3], lane);
+    if ((tid & 7) == 0 && ev < n) lam[ev] = l;
+  }
+  __syncthreads();
+  // eigenvectors of T by inverse iteration: the members of a cluster
+  // (eigenvalues closer than kInvCluster ||T||) are solved in turn by its first
+  // member's thread and orthogonalised against each other
+  if (tid < n) s_start[tid] = (tid == 0 || lam[tid] - lam[tid - 1] > kInvCluster * tn) ? 1 : 0;
+  __syncthreads();
+  const float floor = 1.2e-7f * tn;
+  if (tid < n && s_start[tid]) {
+    int last = tid;
+    while (last + 1 < n && !s_start[last + 1]) ++last;
+    // pivot rows: U[i][i] in Q0, U[i][i+1] in Q1 (NaN when rows i, i+1 were
+    // swapped: then U[i][i+1] = d_{i+1} - lm and U[i][i+2] = e_{i+1})
+    float *Q0 = P0 + tid, *Q1 = P1 + tid;
+    float prev = 0.0f;
+    for (int mm = tid; mm <= last; ++mm) {
+      float *Y = Zs + mm;
+      float lm = lam[mm];                 // members equal to 10 ulps are moved apart
+      const float pert = 10.0f * 1.2e-7f * fabsf(lm);
+      if (mm > tid && lm < prev + pert) lm = prev + pert;
+      prev = lm;
+      for (int j = 0; j < n; ++j) Y[j * ld] = (float)((j * 7919 + mm * 104729) % 1000) * 1.0e-3f - 0.5f;
+      for (int it = 0; it < 2; ++it) {
+        // (T - lm I) y = y: Gaussian elimination with partial pivoting
+        float cd = dd[0] - lm, c1 = ee[0], yc = Y[0];
+        for (int i = 0; i < n - 1; ++i) {
+          const float nd = dd[i + 1] - lm, n1 = i + 1 < n - 1 ? ee[i + 1] : 0.0f, sdn = ee[i];
+          const float yn = Y[(i + 1) * ld];
+          const bool sw = fabsf(sdn) > fabsf(cd);
+          const float num = sw ? cd : sdn, den = sw ? sdn : cd;
+          const float m = den != 0.0f ? __fdividef(num, den) : 0.0f;
+          Q0[i * ld] = sw ? sdn : cd;
+          Q1[i * ld] = sw ? __int_as_float(0x7fc00000) : c1;
+          Y[i * ld] = sw ? yn : yc;
+          const float cn = sw ? c1 - m * nd : nd - m * c1;
+          c1 = sw ? -m * n1 : n1;
+          yc = sw ? yc - m * yn : yn - m * yc;
+          cd = cn;
+        }
+        Q0[(n - 1) * ld] = cd;
+        Q1[(n - 1) * ld] = 0.0f;
+        Y[(n - 1) * ld] = yc;
+        float x1 = 0.0f, x2 = 0.0f;       // back substitution, pivots at least floor
+        for (int i = n - 1; i >= 0; --i) {
+          float d = Q0[i * ld];
+          const float q1 = Q1[i * ld];
+          const bool sw = q1 != q1;
+          const float u1 = sw ? dd[i + 1] - lm : q1;
+          const float u2 = (sw && i + 2 < n) ? ee[i + 1] : 0.0f;
+          if (fabsf(d) < floor) d = d >= 0.0f ? floor : -floor;
+          const float xi = __fdividef(Y[i * ld] - u1 * x1 - u2 * x2, d);
+          Y[i * ld] = xi;
+          x2 = x1; x1 = xi;
+        }
+        for (int q = tid; q < mm; ++q) {  // the cluster's earlier vectors
+          float d = 0.0f;
+          for (int j = 0; j < n; ++j) d += Zs[j * ld + q] * Y[j * ld];
+          for (int j = 0; j < n; ++j) Y[j * ld] -= d * Zs[j * ld + q];
+        }
+        float nrm = 0.0f;
+        for (int j = 0; j < n; ++j) nrm += Y[j * ld] * Y[j * ld];
+        const float inv = nrm > 0.0f ? rsqrtf(nrm) : 0.0f;
+        for (int j = 0; j < n; ++j) Y[j * ld] *= inv;
+      }
+    }
+  }
+  // for back32_kernel: beta of the reflectors, 1 / l_ii and the band of L
+  __syncthreads();
+  float *out = reinterpret_cast<float *>(jb.W);
+  for (int t = tid; t < n; t += nt) { out[t] = bet[t]; out[n + t] = rdg[t]; }
+  for (int t = tid; t < n * kMaxBand; t += nt) out[2 * n + t] = Lb[t];
+  if (tid == 0) *jb.state = 0;
+}
+
+// X = L^{-T} H_0 ... H_{n-3} Z, one warp per column (rows lane, lane + 32, ...
+// of the column in registers), eight columns per CTA
+template <int R>
+__device__ __forceinline__ void back32_column(const EigJob &jb, int c, int lane) {
+  const int n = jb.n, p = jb.p;
+  const float *As = reinterpret_cast<const float *>(jb.A);
+  float *Zs = reinterpret_cast<float *>(jb.A) + (size_t)n * n;
+  const float *bet = reinterpret_cast<const float *>(jb.W), *rdg = bet + n, *Lb = rdg + n;
+  float z[R];
+#pragma unroll
+  for (int t = 0; t < R; ++t) z[t] = lane + 32 * t < n ? Zs[(size_t)(lane + 32 * t) * n + c] : 0.0f;
+  for (int k = n - 3; k >= 0; --k) {
+    const float beta = bet[k];
+    if (beta == 0.0f) continue;
+    float v[R], s = 0.0f;
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const int r = lane + 32 * t;
+      v[t] = r > k && r < n ? As[(size_t)k * n + r] : 0.0f;
+      s += v[t] * z[t];
+    }
+    s = beta * warp_sum_f(s);
+#pragma unroll
+    for (int t = 0; t < R; ++t) z[t] -= s * v[t];
+  }
+  // backward substitution: row i's lane owns x_i and sends it to the rows
+  // i - 1 .. i - p it enters (column i of L: Lb[i][d] = L[i][i - d])
+#pragma unroll
+  for (int t = R - 1; t >= 0; --t) {
+    for (int l = 31; l >= 0; --l) {
+      const int i = 32 * t + l;
+      if (i >= n) continue;
+      const float x = __shfl_sync(0xffffffffu, z[t], l) * rdg[i];
+      if (lane == l) z[t] = x;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {         // rows of this register and the one below
+        if (t - u < 0) continue;
+        const int d = i - (lane + 32 * (t - u));
+        if (d >= 1 && d <= p) z[t - u] -= Lb[i * kMaxBand + d] * x;
+      }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < R; ++t)
+    if (lane + 32 * t < n) jb.X[(size_t)(lane + 32 * t) * n + c] = (double)z[t];
+}
+__global__ void __launch_bounds__(256) back32_kernel(EigJob *jobs, int allow_fast) {
+  const EigJob jb = jobs[blockIdx.y];
+  const int n = jb.n, c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (!allow_fast || n <= kFastMaxN || c >= n || *jb.state != 0) return;
+  if (n <= 256) back32_column<8>(jb, c, lane);
+  else if (n <= 512) back32_column<16>(jb, c, lane);
+  else back32_column<32>(jb, c, lane);
+}
+
 // ---- fast route: dense FP64 products C = op(A) B (+ D), many CTAs ----
 struct GemmJob {
   int n, transA;
@@ -750,8 +1108,10 @@ __global__ void __launch_bounds__(32) refine_kernel(EigJob *jobs) {
 
 // Refinement step, second half: the correction E (into W), E_ii = r_ii / 2,
 // E_ij = (s_ij + lambda_j r_ij) / (lambda_j - lambda_i) for separated pairs
-// and r_ij / 2 within a cluster (r = I - G), one element per thread.
-__global__ void correction_kernel(EigJob *jobs) {
+// and r_ij / 2 within a cluster (r = I - G), one element per thread. With
+// polish, r_ij / 2 everywhere: X is only made M-orthonormal, which does not
+// divide the rounding of S by the gaps.
+__global__ void correction_kernel(EigJob *jobs, int polish) {
   const EigJob jb = jobs[blockIdx.y];
   if (*jb.state != 0) return;
   const int n = jb.n;
@@ -764,7 +1124,7 @@ __global__ void correction_kernel(EigJob *jobs) {
     e = 0.5 * (1.0 - g);
   } else {
     const double d = lam[j] - lam[i];
-    e = fabs(d) > jb.sc[1] ? (jb.S[t] - lam[j] * g) / d : -0.5 * g;
+    e = !polish && fabs(d) > jb.sc[1] ? (jb.S[t] - lam[j] * g) / d : -0.5 * g;
   }
   jb.W[t] = e;
 }
@@ -782,12 +1142,12 @@ __global__ void __launch_bounds__(1024) cluster_kernel(EigJob *jobs, int parity)
   double *X = parity ? jb.Xn : jb.X;
   double *S = jb.S;
   __shared__ int np_s, pi_s[kMaxPairs], pj_s[kMaxPairs];
-  __shared__ double c_sh, s_sh, dg[kFastMaxN];
+  __shared__ double c_sh, s_sh, dg[kBigMaxN];
   for (int i = tid; i < n; i += nt) dg[i] = S[(size_t)i * n + i];
   __syncthreads();
   // the pair list in a fixed order ((i, j) lexicographic: row counts, a
   // prefix sum, then each row writes its own pairs), so results are reproducible
-  __shared__ int cnt_s[kFastMaxN], off_s[kFastMaxN];
+  __shared__ int cnt_s[kBigMaxN], off_s[kBigMaxN];
   const double thr = kClusterRel * jb.sc[0];
   if (tid < n) {
     int c = 0;
@@ -1040,28 +1400,20 @@ __global__ void __launch_bounds__(1024) finish_kernel(EigJob *jobs, int parity) 
   __syncthreads();
   // eigenvalues ranked and magnitudes compared as integers (a monotone map
   // of the FP64 bit patterns: GB300's FP64 pipe is slow)
-  __shared__ unsigned long long key[kFastMaxN];
+  __shared__ unsigned long long key[kBigMaxN];
   auto order_key = [](double v) -> unsigned long long {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
   };
-  if (n <= kFastMaxN)
-    for (int i = tid; i < n; i += nt) key[i] = order_key(Lam[(size_t)i * n + i]);
+  for (int i = tid; i < n; i += nt) key[i] = order_key(Lam[(size_t)i * n + i]);
   __syncthreads();
   for (int i = tid; i < n; i += nt) {
-    double li = Lam[(size_t)i * n + i];
+    const double li = Lam[(size_t)i * n + i];
     int rank = 0;
-    if (n <= kFastMaxN) {
-      const unsigned long long ki = key[i];
-      for (int j = 0; j < n; ++j) {
-        const unsigned long long kj = key[j];
-        rank += (kj < ki || (kj == ki && j < i)) ? 1 : 0;
-      }
-    } else {
-      for (int j = 0; j < n; ++j) {
-        double lj = Lam[(size_t)j * n + j];
-        if (lj < li || (lj == li && j < i)) ++rank;
-      }
+    const unsigned long long ki = key[i];
+    for (int j = 0; j < n; ++j) {
+      const unsigned long long kj = key[j];
+      rank += (kj < ki || (kj == ki && j < i)) ? 1 : 0;
     }
     int imax = 0;
     unsigned long long vmax = 0ull;
@@ -1164,12 +1516,13 @@ igafd_status igafd_setup_pencils_eig(igafd_patch *P, cudaStream_t s, const doubl
   }
   EigJob hjobs[3];
   size_t off = 0;
-  int max_n = 0, fast_jobs = 0;
+  int max_n = 0, fast_jobs = 0, big_jobs = 0;
   for (int u = 0; u < nj; ++u) {
     const int k = dir_of[u];
     int n = P->n[k];
     max_n = n > max_n ? n : max_n;
-    fast_jobs += n <= kFastMaxN;
+    fast_jobs += p < kMaxBand;
+    big_jobs += n > kFastMaxN;
     size_t nn = (size_t)n * n;
     EigJob &j = hjobs[u];
     double *w = P->eig_work + off;
@@ -1208,6 +1561,18 @@ igafd_status igafd_setup_pencils_eig(igafd_patch *P, cudaStream_t s, const doubl
     }
     tri32_kernel<<<nj, 1024, smem32, s>>>(djobs, allow_fast);
     IGAFD_LAUNCHED(1);
+    if (big_jobs > 0 && allow_fast) {
+      const size_t big = big32_smem_floats(kBigMaxN) * sizeof(float);
+      static std::atomic<unsigned long long> big_set{0};
+      if (!(big_set.load() & bit)) {
+        IGAFD_CUDA(cudaFuncSetAttribute(big32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big));
+        big_set.fetch_or(bit);
+      }
+      big32_kernel<<<nj, 1024, big32_smem_floats(max_n) * sizeof(float), s>>>(djobs, allow_fast);
+      back32_kernel<<<dim3((max_n + 7) / 8, nj), 256, 0, s>>>(djobs, allow_fast);
+      IGAFD_LAUNCHED(2);
+      IGAFD_CUDA(cudaGetLastError());
+    }
   }
   int parity = 0;
   if (allow_fast && fast_jobs > 0) {
@@ -1234,12 +1599,16 @@ igafd_status igafd_setup_pencils_eig(igafd_patch *P, cudaStream_t s, const doubl
       return IGAFD_OK;
     };
     // an FP32 start is refined to the FP64 level in two steps; the third
-    // leaves margin below the acceptance test
-    for (int it = 0; it < 3; ++it) {
+    // leaves margin below the acceptance test. Larger pencils start further
+    // off (the FP32 error grows with ||K~|| over the eigenvalues' gaps) and
+    // end with a polishing step: at their noise level a step perturbs the
+    // orthogonality by 2^-53 ||K~|| over the smallest gap (1e-12 at n = 250).
+    const int steps = big_jobs == 0 ? 3 : max_n <= 512 ? 5 : 7;
+    for (int it = 0; it < steps; ++it) {
       IGAFD_TRY(products());
       refine_kernel<<<dim3(nmax, nj), 32, 0, s>>>(djobs);
       IGAFD_LAUNCHED(1);
-      correction_kernel<<<dim3((nmax * nmax + 255) / 256, nj), 256, 0, s>>>(djobs);
+      correction_kernel<<<dim3((nmax * nmax + 255) / 256, nj), 256, 0, s>>>(djobs, big_jobs > 0 && it == steps - 1);
       IGAFD_LAUNCHED(1);
       GemmBatch b3{};
       for (int u = 0; u < nj; ++u) {
@@ -1309,8 +1678,8 @@ igafd_status igafd_setup_pencils_eig(igafd_patch *P, cudaStream_t s, const doubl
   for (int k = 0; k < dim; ++k) {
     const int u = job_of[k];
     P->eig_used[k] = hstate[u];
-    P->eig_check[k][0] = allow_fast && P->n[k] <= kFastMaxN ? hsc[u][2] : 0.0;
-    P->eig_check[k][1] = allow_fast && P->n[k] <= kFastMaxN ? hsc[u][3] : 0.0;
+    P->eig_check[k][0] = allow_fast ? hsc[u][2] : 0.0;
+    P->eig_check[k][1] = allow_fast ? hsc[u][3] : 0.0;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

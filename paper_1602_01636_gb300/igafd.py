@@ -536,7 +536,7 @@ class Patch:
         return k.value, lo.value, hi.value
 
     def set_eig_route(self, route):
-        """0: FP32 Jacobi + FP64 refinement where n_k <= 128 (default); 1: FP64 Jacobi.
+        """0: FP32 start + FP64 refinement (default); 1: FP64 Jacobi.
         Takes effect at the next setup_prec()."""
         _check(lib().igafd_set_eig_route(self.h, int(route)), "set_eig_route")
 
