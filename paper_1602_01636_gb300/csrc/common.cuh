@@ -128,7 +128,7 @@ struct igafd_patch {
   double *coef;                 // [2 * IGAFD_COEF_CAP]: alpha_k, beta_k of the last solve
   double *host_scal;            // pinned mirror of scal
   FDMixed *mixed;
-  FDSplit *split;               // null: n_k > 128 in some direction
+  FDSplit *split;               // null: n_k > 256 in some direction
   double *wK[3], *wM[3];        // span scalings of the pencils (device, null = unscaled)
   int fd_fused;                 // 1: fused tensor-core FD (3 kernels) when n_k <= 128
   int fd_fused_op[3];           // the same per operand type (TF32, BF16, FP16), set by the autotuner
@@ -179,7 +179,7 @@ igafd_status igafd_adi_apply(igafd_patch *P, const double *r, double *z, cudaStr
 // FD apply; kernels do nothing while *done_flag != 0 (done_flag may be null)
 igafd_status igafd_fd64_apply(igafd_patch *P, const double *r, double *z, cudaStream_t s,
                               double *done_flag);
-// FP64 FD on the tensor cores (every n_k <= 128)
+// FP64 FD on the tensor cores (every n_k <= 256)
 bool igafd_fd_split_shape(const igafd_patch *P);
 igafd_status igafd_fd_split_init(igafd_patch *P, cudaStream_t s);
 void igafd_fd_split_free(igafd_patch *P);

@@ -1603,7 +1603,7 @@ igafd_status igafd_setup_pencils_eig(igafd_patch *P, cudaStream_t s, const doubl
     // off (the FP32 error grows with ||K~|| over the eigenvalues' gaps) and
     // end with a polishing step: at their noise level a step perturbs the
     // orthogonality by 2^-53 ||K~|| over the smallest gap (1e-12 at n = 250).
-    const int steps = big_jobs == 0 ? 3 : max_n <= 512 ? 5 : 7;
+    const int steps = big_jobs > 0 ? 5 : 3;
     for (int it = 0; it < steps; ++it) {
       IGAFD_TRY(products());
       refine_kernel<<<dim3(nmax, nj), 32, 0, s>>>(djobs);

@@ -1,4 +1,4 @@
-// FP64 fast-diagonalization apply on the tensor cores, for n_k <= 128.
+// FP64 fast-diagonalization apply on the tensor cores, for n_k <= 256.
 //
 // GB300 issues two FP64 FMAs per clock per SM (1.26 TFLOP/s in all), so the
 // 12 n^4 FLOP of the six mode products take 2.6 ms at n = 128 on the FP64
@@ -24,7 +24,7 @@
 // executed (each would issue at the 2-per-clock rate).
 //
 // Measured: 170 us per apply at n = 128 (SIMT: 3.10 ms), 95 us at (95, 61, 77)
-// (SIMT: 0.98 ms). A pass at n = 128 is bound by integer instructions (64
+// (SIMT: 0.98 ms), 1.23 ms at n = 192 (SIMT: 13.8 ms). A pass at n = 128 is bound by integer instructions (64
 // lanes per clock per SM, conversions 16): 20 us, of which reading and
 // splitting the rows 6 us, the MMAs with the summation of their accumulators
 // 9 us (the MMAs alone 5), the last rounding 2.5 us; about 6 us pass between
@@ -57,7 +57,6 @@ constexpr int kM = 128;                 // rows per CTA (MMA M, TMEM lanes)
 constexpr int kThreads = 512;           // 4 warps per lane quarter
 constexpr int kWarps = kThreads / 32;
 constexpr int kSlices = 6;              // digits per operand
-constexpr int kTrans = 16 * 32 * 17 * 8;// bytes of the transposition buffers
 constexpr long long kSpin = 1ll << 26;  // bounded waits
 // X + kBias = sum_s (digit_s + 512) 1024^(5-s): every 10-bit field is then the
 // digit plus 512
@@ -226,10 +225,19 @@ __device__ __forceinline__ double round_fixed(long long T, int E, double lam, bo
 // columns and half the shared memory each), so one's MMAs and the start of the
 // next launch overlap the other's integer work.
 constexpr int acc_cols(int KP) { return KP > 64 ? 64 : 32; }
+// With K > 128 the rows are split and multiplied in two parts (the first 128
+// terms, then the rest, on the same row exponents) whose groups add up in the
+// 64-bit sums; a CTA then takes at most 64 columns, so that B's digits of both
+// parts fit.
+constexpr int part_terms(int KP) { return KP > 128 ? 128 : KP; }
+constexpr int b_rows(int KP) { return KP > 128 ? 64 : kM; }
 constexpr int ctas_per_sm(int KP) { return KP > 64 ? 1 : 2; }
 // slices of B fetched before the input is read (the rest of B's shared memory
 // holds the transposition buffers until then)
-constexpr int first_slices(int KP) { return KP > 64 ? 3 : 1; }
+constexpr int first_slices(int KP) { return KP > 128 ? kSlices : KP > 64 ? 3 : 1; }
+// doubles per row of a transposition buffer, and its bytes for all warps
+constexpr int trans_cols(int KP) { return KP > 128 ? 8 : 17; }
+constexpr int trans_bytes(int KP) { return 16 * 32 * trans_cols(KP) * 8; }
 template <int KP, bool LAM>
 __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(SplitArgs a) {
   extern __shared__ unsigned char smem_raw[];
@@ -242,18 +250,30 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
   const int n0 = (int)blockIdx.y * a.NT;
   const int NTc = a.Np - n0 < a.NT ? a.Np - n0 : a.NT;     // columns of this CTA
   constexpr int nkc = (KP + 63) / 64;                      // 64-wide K chunks
-  constexpr int KS = KP / 16;                              // MMAs per digit product
-  constexpr int scols = KP / 2;                            // TMEM columns per slice of A
+  constexpr int KA = part_terms(KP);                       // terms of the first part
+  constexpr int KR = KP - KA;                              // and of the second
+  constexpr int scols = KA / 2;                            // TMEM columns per slice of A
   constexpr int dbase = kSlices * scols;                   // two accumulators follow
-  constexpr int per = Steps<KP>::kCount;                   // steps per column block
   constexpr int kNS = acc_cols(KP), kFirst = first_slices(KP);
   constexpr int kTmem = dbase + 2 * kNS > 256 ? 512 : 256; // allocated columns
-  // B in shared memory: [slice][chunk][128 rows][128 B] (row strides fixed, so
+  // B in shared memory: [slice][chunk][128 (64) rows][128 B] (row strides fixed, so
   // that descriptors are constants apart from the column block)
-  constexpr int kChunk = kM * 128;
+  constexpr int kChunk = b_rows(KP) * 128;
   constexpr int slice_bytes = nkc * kChunk;
   const int nsub = (NTc + kNS - 1) / kNS;
 
+  // Already converged when this launch begins (the flag only rises within a
+  // solve): leave before TMEM and B's digits are taken, still in stream order.
+  if (a.done) {
+    if (tid == 0) s_fail = *(volatile const double *)a.done != 0.0;
+    __syncthreads();
+    if (s_fail) {
+      pdl_wait();
+      pdl_trigger();
+      return;
+    }
+    __syncthreads();
+  }
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bar_b[i], 1);
@@ -300,39 +320,41 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     return;
   }
 
-  // ---- A: this thread's row (lane 32 q + lane) and K range [kq KQ, kq KQ + KQ) ----
+  // ---- A: this thread's row (lane 32 q + lane) and K range [kq KQ, kq KQ + KQ)
+  // of a part ----
   const int q = warp & 3, kq = warp >> 2;
-  constexpr int KQ = KP / 4;                             // 8, 16, 24 or 32
+  constexpr int KQ = KA / 4;                               // 8, 16, 24 or 32
   const int lrow = q * 32 + lane;
   const long long m = (long long)blockIdx.x * kM + lrow;
   const bool row_ok = m < a.M;
   const long long hi = row_ok ? m / a.F : 0, lo = row_ok ? m - hi * a.F : 0;
   const int k0 = kq * KQ;
   const uint32_t lanes = (uint32_t)(q * 32) << 16;
-  int ea;
-  {
-    double x[KQ];
+  auto load_row = [&](int kb, double (&x)[KQ]) {           // terms kb + k0 ..
     if (a.in_k != 1) {
-      const double *src = a.in + hi * a.in_hi + lo * a.in_lo + (long long)k0 * a.in_k;
+      const double *src = a.in + hi * a.in_hi + lo * a.in_lo + (long long)(kb + k0) * a.in_k;
 #pragma unroll
       for (int i = 0; i < KQ; ++i)
-        x[i] = (row_ok && k0 + i < a.K) ? __ldg(src + (long long)i * a.in_k) : 0.0;
+        x[i] = (row_ok && kb + k0 + i < a.K) ? __ldg(src + (long long)i * a.in_k) : 0.0;
     } else {
-      // rows contiguous in K: a warp reads runs of two rows at a time and
-      // transposes through its own buffer (in the part of shared memory that
-      // the later digits of B take afterwards)
-      constexpr int HP = (KQ + 15) / 16;                 // pieces of 16 elements
-      double *buf = reinterpret_cast<double *>(sB + (size_t)kFirst * slice_bytes) + warp * 32 * 17;
+      // rows contiguous in K: a warp reads runs of several rows at a time and
+      // transposes through its own buffer (up to K = 128 in the part of shared
+      // memory that the later digits of B take afterwards)
+      constexpr int PW = KP > 128 ? 8 : 16;                // elements of a row per piece
+      constexpr int TC = trans_cols(KP), HP = (KQ + PW - 1) / PW, RW = 32 / PW;
+      double *buf = reinterpret_cast<double *>(sB + (size_t)kFirst * slice_bytes) + warp * 32 * TC;
       const long long base = row_ok ? hi * a.in_hi + lo * a.in_lo : -1;
-      const int cc = lane & 15;
-      double y[HP][16];
+      const int cc = lane % PW;
+      // the 8-wide buffer is unpadded: its columns are exchanged by row instead
+      auto at = [&](int r, int c) { return r * TC + (TC == 8 ? c ^ (r & 7) : c); };
+      double y[HP][PW];
 #pragma unroll
       for (int h = 0; h < HP; ++h) {
 #pragma unroll
-        for (int t = 0; t < 16; ++t) {
-          const int k = k0 + 16 * h + cc;
-          const long long b = __shfl_sync(0xffffffffu, base, 2 * t + (lane >> 4));
-          const bool ok = b >= 0 && 16 * h + cc < KQ && k < a.K;
+        for (int t = 0; t < PW; ++t) {
+          const int k = kb + k0 + PW * h + cc;
+          const long long b = __shfl_sync(0xffffffffu, base, RW * t + lane / PW);
+          const bool ok = b >= 0 && PW * h + cc < KQ && k < a.K;
           y[h][t] = ok ? __ldg(a.in + b + k) : 0.0;
         }
       }
@@ -340,26 +362,23 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
       for (int h = 0; h < HP; ++h) {
         __syncwarp();
 #pragma unroll
-        for (int t = 0; t < 16; ++t) buf[(2 * t + (lane >> 4)) * 17 + cc] = y[h][t];
+        for (int t = 0; t < PW; ++t) buf[at(RW * t + lane / PW, cc)] = y[h][t];
         __syncwarp();
 #pragma unroll
-        for (int t = 0; t < 16; ++t)
-          if (16 * h + t < KQ) x[16 * h + t] = buf[lane * 17 + t];
+        for (int t = 0; t < PW; ++t)
+          if (PW * h + t < KQ) x[PW * h + t] = buf[at(lane, t)];
       }
+      __syncwarp();
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (LAM && row_ok && (lane & 15) == 0) {              // the divide's table, used last
-      const double *t = a.inv_lam + hi * a.out_hi + lo * a.out_lo + (long long)n0 * a.out_n;
-      for (int n = kq; n < NTc && n0 + n < a.N; n += 4)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(t + (long long)n * a.out_n));
-    }
-    int em = 1;
+  };
+  auto largest = [&](const double (&x)[KQ], int em) {
 #pragma unroll
     for (int i = 0; i < KQ; ++i) em = max(em, exp_field((uint32_t)__double2hiint(x[i])));
-    s_ea[kq][lrow] = (unsigned short)em;
-    __syncthreads();
-    if (tid == 0) load_slices(kFirst, kSlices, &bar_b[1]);
-    ea = max(max((int)s_ea[0][lrow], (int)s_ea[1][lrow]), max((int)s_ea[2][lrow], (int)s_ea[3][lrow]));
+    return em;
+  };
+  // the digits of a part into TMEM
+  auto put_digits = [&](const double (&x)[KQ], int ea) {
     uint32_t w1[KQ], w0[KQ];
 #pragma unroll
     for (int i = 0; i < KQ; ++i) biased_fixed<58>(x[i], ea, w1[i], w0[i]);
@@ -381,10 +400,30 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     put(3, std::integral_constant<int, 2>{}, w0);
     put(4, std::integral_constant<int, 1>{}, w0);
     put(5, std::integral_constant<int, 0>{}, w0);
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+  };
+  int ea;
+  {
+    double x[KQ];
+    int em = 1;
+    if constexpr (KR > 0) {                                // the second part's exponents too
+      load_row(KA, x);
+      em = largest(x, em);
+    }
+    load_row(0, x);
+    if (LAM && row_ok && (lane & 15) == 0) {               // the divide's table, used last
+      const double *t = a.inv_lam + hi * a.out_hi + lo * a.out_lo + (long long)n0 * a.out_n;
+      for (int n = kq; n < NTc && n0 + n < a.N; n += 4)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(t + (long long)n * a.out_n));
+    }
+    s_ea[kq][lrow] = (unsigned short)largest(x, em);
+    __syncthreads();
+    if (kFirst < kSlices && tid == 0) load_slices(kFirst, kSlices, &bar_b[1]);
+    ea = max(max((int)s_ea[0][lrow], (int)s_ea[1][lrow]), max((int)s_ea[2][lrow], (int)s_ea[3][lrow]));
+    put_digits(x, ea);
   }
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
 
   // ---- digit products. A step's MMAs are issued by one elected lane of warp
   // step mod 16, while the others sum the step before. (Elected by elect.sync,
@@ -395,11 +434,13 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
   const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
   const uint64_t b0 = sw128_desc(smem_u32(sB));
   bool ok = true;
-  auto issue = [&](auto step, int sub, int st) {           // one warp
-    constexpr int i = decltype(step)::value;
-    constexpr Step p = Steps<KP>::at(i);
+  // K terms of part `part` (KT of them, from chunk c0), group and chunks of step i
+  auto issue = [&](auto part, auto step, int sub, int st) {   // one warp
+    constexpr int i = decltype(step)::value, part_ = decltype(part)::value;
+    constexpr int KT = part_ ? KR : KA, KS = KT / 16, kc0 = part_ ? KA / 64 : 0;
+    constexpr Step p = Steps<KT>::at(i);
     const int buf = st & 1;
-    if (i == 0 && sub == 0) ok = ok && wait_on(&bar_b[0], 0, &s_fail);
+    if (i == 0 && sub == 0 && part_ == 0) ok = ok && wait_on(&bar_b[0], 0, &s_fail);
     if (p.g >= kFirst && sub == 0) ok = ok && wait_on(&bar_b[1], 0, &s_fail);
     if (st >= 2) ok = ok && wait_on(&bar_empty[buf], (uint32_t)(((st >> 1) - 1) & 1), &s_fail);
     ok = __all_sync(0xffffffffu, ok);
@@ -423,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
               "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
               " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
               "r"(tm + (uint32_t)(sl * scols + ks * 8)),
-              "l"(bs + (uint64_t)((ks >> 2) * (kChunk >> 4) + (ks & 3) * 2)), "r"(idesc), "r"(acc));
+              "l"(bs + (uint64_t)(((ks >> 2) + kc0) * (kChunk >> 4) + (ks & 3) * 2)), "r"(idesc), "r"(acc));
         }
       }
       asm volatile(
@@ -433,20 +474,22 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     }
     __syncwarp();
   };
-  if (warp == 0) issue(std::integral_constant<int, 0>{}, 0, 0);
   // ---- accumulators to integers, rounded once ----
   constexpr int C = kNS / 4;                               // columns per thread in a block
   const bool bad_row = ea == 0x7ff;
   const long long ob = hi * a.out_hi + lo * a.out_lo;
+  constexpr int kTop = KR > 0 ? 37 : 38;                   // weight of group 0 in T
   int st = 0;
+  if (warp == 0) issue(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{}, 0, 0);
   for (int sub = 0; sub < nsub; ++sub) {
     long long T[C];
-    auto sum = [&](auto step) {
-      constexpr int i = decltype(step)::value;
-      constexpr int g = Steps<KP>::at(i).g;
+    auto sum = [&](auto part, auto step) {
+      constexpr int i = decltype(step)::value, part_ = decltype(part)::value;
+      constexpr int KT = part_ ? KR : KA, per = Steps<KT>::kCount;
+      constexpr int g = Steps<KT>::at(i).g;
       const int buf = st & 1;
-      if (warp == ((st + 1) & (kWarps - 1)) && (i + 1 < per || sub + 1 < nsub))
-        issue(std::integral_constant<int, (i + 1) % per>{}, i + 1 < per ? sub : sub + 1, st + 1);
+      if (warp == ((st + 1) & (kWarps - 1)) && (i + 1 < per || (KR == 0 && sub + 1 < nsub)))
+        issue(part, std::integral_constant<int, (i + 1) % per>{}, i + 1 < per ? sub : sub + 1, st + 1);
       ok = ok && wait_on(&bar_full[buf], (uint32_t)((st >> 1) & 1), &s_fail);
       ok = __all_sync(0xffffffffu, ok);
       ++st;
@@ -474,25 +517,40 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_empty[buf]);
-      // T in units of 2^12 of group 5: |G_0| 2^38 <= 2^62; what is dropped of
-      // groups 4 and 5 is of the order of the groups not computed
+      // T in units of 2^12 (2^13 with two parts) of group 5: a part's |G_0|
+      // 2^38 <= 2^62; what is dropped of groups 4 and 5 is of the order of the
+      // groups not computed
 #pragma unroll
       for (int c = 0; c < C; ++c) {
         const int G = __float2int_rn(__uint_as_float(v[c]));
-        if (g == 0) T[c] = (long long)G << 38;
-        else if (g < 4) T[c] += (long long)G * (1 << (g > 0 && g < 4 ? 38 - 10 * g : 0));
-        else T[c] += (long long)(g == 4 ? (G + 2) >> 2 : (G + 2048) >> 12);
+        constexpr int w = kTop - 10 * g;                   // 2^w: the group's weight
+        if (g == 0) T[c] = (part_ ? T[c] : 0) + ((long long)G << kTop);
+        else if (w >= 0) T[c] += (long long)G * (1 << (w >= 0 && w < 31 ? w : 0));
+        else T[c] += (long long)((G + (1 << (w < 0 ? -w - 1 : 0))) >> (w < 0 ? -w : 0));
       }
     };
-    sum(std::integral_constant<int, 0>{});
-    sum(std::integral_constant<int, 1>{});
-    sum(std::integral_constant<int, 2>{});
-    sum(std::integral_constant<int, 3>{});
-    sum(std::integral_constant<int, 4>{});
-    sum(std::integral_constant<int, 5>{});
-    if constexpr (per == 8) {
-      sum(std::integral_constant<int, 6>{});
-      sum(std::integral_constant<int, 7>{});
+    auto sum_part = [&](auto part) {
+      sum(part, std::integral_constant<int, 0>{});
+      sum(part, std::integral_constant<int, 1>{});
+      sum(part, std::integral_constant<int, 2>{});
+      sum(part, std::integral_constant<int, 3>{});
+      sum(part, std::integral_constant<int, 4>{});
+      sum(part, std::integral_constant<int, 5>{});
+      if constexpr (Steps<decltype(part)::value ? KR : KA>::kCount == 8) {
+        sum(part, std::integral_constant<int, 6>{});
+        sum(part, std::integral_constant<int, 7>{});
+      }
+    };
+    sum_part(std::integral_constant<int, 0>{});
+    if constexpr (KR > 0) {                                // (one column block)
+      constexpr std::integral_constant<int, 1> second{};
+      double x[KQ];
+      load_row(KA, x);
+      __syncthreads();                                     // every MMA on the first digits is done
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      put_digits(x, ea);
+      if (warp == (st & (kWarps - 1))) issue(second, std::integral_constant<int, 0>{}, 0, st);
+      sum_part(second);
     }
     if (!ok || !row_ok) continue;
     const int nl0 = sub * kNS + kq * C;                  // this thread's first column, and how many
@@ -504,7 +562,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     bool slow = bad_row;
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      const double y = round_fixed<LAM>(T[c], ea + (int)s_eb[(nl0 + c) & (kM - 1)] - 2099, lam[c], slow);
+      const double y = round_fixed<LAM>(T[c], ea + (int)s_eb[(nl0 + c) & (kM - 1)] - 2061 - kTop, lam[c], slow);
       if (c < ncol) a.out[o0 + c * a.out_n] = y;
     }
     if (slow) {                                          // rare: again, one by one
@@ -513,7 +571,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
         if (c < ncol)
           a.out[o0 + c * a.out_n] =
               bad_row ? __longlong_as_double(0x7ff8000000000000ll)
-                      : round_slow(T[c], ea + (int)s_eb[nl0 + c] - 2099, lam[c]);
+                      : round_slow(T[c], ea + (int)s_eb[nl0 + c] - 2061 - kTop, lam[c]);
     }
   }
   if (!ok) s_fail = 1;
@@ -546,11 +604,11 @@ struct ImgJob {
 struct ImgBatch {
   ImgJob j[6];
 };
-__global__ void __launch_bounds__(128) split_image_kernel(ImgBatch b) {
+__global__ void __launch_bounds__(256) split_image_kernel(ImgBatch b) {
   const ImgJob J = b.j[blockIdx.y];
   const int r = blockIdx.x, k = threadIdx.x;
   if (r >= J.Np) return;
-  __shared__ int s_e[4];
+  __shared__ int s_e[8];
   const int nkc = (J.Kp + 63) >> 6;
   double d = 0.0;
   if (r < J.n && k < J.n) d = J.transpose ? J.U[(size_t)k * J.n + r] : J.U[(size_t)r * J.n + k];
@@ -558,7 +616,7 @@ __global__ void __launch_bounds__(128) split_image_kernel(ImgBatch b) {
   for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
   if ((k & 31) == 0) s_e[k >> 5] = e;
   __syncthreads();
-  e = max(max(s_e[0], s_e[1]), max(s_e[2], s_e[3]));
+  for (int w = 0; w < 8; ++w) e = max(e, s_e[w]);
   if (k == 0) J.eb[r] = e;
   if (k >= nkc * 64) return;
   uint32_t w1, w0;
@@ -578,8 +636,8 @@ __global__ void __launch_bounds__(128) split_image_kernel(ImgBatch b) {
 int pad(int n, int to) { return (n + to - 1) / to * to; }
 
 size_t pass_smem(int Kp) {
-  const size_t slice = (size_t)((Kp + 63) / 64) * kM * 128;
-  const size_t a = kSlices * slice, b = first_slices(Kp) * slice + kTrans;
+  const size_t slice = (size_t)((Kp + 63) / 64) * b_rows(Kp) * 128;
+  const size_t a = kSlices * slice, b = first_slices(Kp) * slice + trans_bytes(Kp);
   return 1024 + (a > b ? a : b);
 }
 
@@ -592,7 +650,7 @@ struct FDSplit {
 
 bool igafd_fd_split_shape(const igafd_patch *P) {
   for (int k = 0; k < P->dim; ++k)
-    if (P->n[k] > 128) return false;
+    if (P->n[k] > 256) return false;
   return true;
 }
 
@@ -621,7 +679,7 @@ igafd_status igafd_fd_split_init(igafd_patch *P, cudaStream_t s) {
       J.eb = P->split->eb[k][d];
       rows = J.Np > rows ? J.Np : rows;
     }
-  split_image_kernel<<<dim3(rows, jobs), 128, 0, s>>>(b);
+  split_image_kernel<<<dim3(rows, jobs), 256, 0, s>>>(b);
   IGAFD_LAUNCHED(1);
   IGAFD_CUDA(cudaGetLastError());
   return IGAFD_OK;
@@ -653,20 +711,21 @@ static igafd_status launch_pass(igafd_patch *P, int k, int dir, SplitArgs a, cud
   const long long tiles = (a.M + kM - 1) / kM;
   int parts = 1;
   while (parts < 8 && tiles * parts * 2 <= P->num_sms && pad(a.Np, 32 * parts) / parts > 16) parts *= 2;
+  if (a.Kp > 128) parts = parts < (a.Np + 63) / 64 ? (a.Np + 63) / 64 : parts;
   a.NT = pad((a.Np + parts - 1) / parts, 16);
   parts = (a.Np + a.NT - 1) / a.NT;
   const size_t smem = pass_smem(a.Kp);
   using Kern = void (*)(SplitArgs);
-  static const Kern kerns[4][2] = {{split_pass_kernel<32, false>, split_pass_kernel<32, true>},
-                                   {split_pass_kernel<64, false>, split_pass_kernel<64, true>},
-                                   {split_pass_kernel<96, false>, split_pass_kernel<96, true>},
-                                   {split_pass_kernel<128, false>, split_pass_kernel<128, true>}};
+#define IGAFD_SPLIT(K) {split_pass_kernel<K, false>, split_pass_kernel<K, true>}
+  static const Kern kerns[8][2] = {IGAFD_SPLIT(32),  IGAFD_SPLIT(64),  IGAFD_SPLIT(96),  IGAFD_SPLIT(128),
+                                   IGAFD_SPLIT(160), IGAFD_SPLIT(192), IGAFD_SPLIT(224), IGAFD_SPLIT(256)};
+#undef IGAFD_SPLIT
   static std::atomic<unsigned long long> attr_set{0};
   const unsigned long long bit = 1ull << (P->dev & 63);
   if (!(attr_set.load() & bit)) {
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 16; ++i)
       IGAFD_CUDA(cudaFuncSetAttribute(kerns[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)pass_smem(128)));
+                                      (int)pass_smem(32 * (i / 2 + 1))));
     attr_set.fetch_or(bit);
   }
   IGAFD_CUDA(igafd_launch(kerns[a.Kp / 32 - 1][a.inv_lam ? 1 : 0], dim3((unsigned)tiles, (unsigned)parts),

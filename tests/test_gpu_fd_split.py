@@ -1,4 +1,4 @@
-"""The FP64 FD on the tensor cores (every n_k <= 128) against mode products in
+"""The FP64 FD on the tensor cores (every n_k <= 256) against mode products in
 80-bit arithmetic with the library's own U_k and D_k, so that only the
 products' rounding is seen.
 
@@ -18,7 +18,9 @@ pytestmark = pytest.mark.gpu
 # tile edges: K padded to 32 (one and two 64-wide chunks), columns to 16 and in
 # blocks of 64, rows in tiles of 128, column splits of small problems
 CASES = [(3, (32, 32, 32), 3), (3, (33, 31, 65), 2), (3, (64, 17, 97), 3), (3, (127, 3, 128), 1),
-         (3, (2, 1, 5), 1), (3, (128, 112, 40), 3), (2, (128, 17), 3), (2, (1, 129 - 1), 2), (2, (96, 95), 4)]
+         (3, (2, 1, 5), 1), (3, (128, 112, 40), 3), (2, (128, 17), 3), (2, (1, 129 - 1), 2), (2, (96, 95), 4),
+         # two parts (K > 128): every padded length, one and several column blocks
+         (2, (129, 160), 3), (3, (150, 24, 20), 2), (2, (193, 40), 2), (2, (256, 225), 3), (3, (10, 161, 9), 3)]
 
 
 def reference(patch, r):
