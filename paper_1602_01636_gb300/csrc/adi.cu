@@ -11,10 +11,12 @@
 // into shared memory with coalesced loads (direction 1: kL whole rows, which
 // are contiguous; directions 2 and 3: kL consecutive i_1 at every position
 // along the line), forms the products with all its threads, solves with one
-// thread per line (forward and backward substitution, p terms each), and
-// stores coalesced. Per iteration four such kernels run:
+// thread per line (FP32) or one for each end of it (FP64), and stores
+// coalesced. Per iteration four such kernels run:
 //   dir 2: u_j = (M2^{-1} K2) s_{j-1}
 //   dir 1: s*_j = (K1 + w M1)^{-1} (r~ - (K1 - w M1) s_{j-1} - 2 M1 (u_j + v_j))
+//          (in FP64 as s*_j = (K1 + w M1)^{-1} (r~ + 2 M1 (w s_{j-1} - u_j - v_j)) - s_{j-1}:
+//          one banded product instead of two)
 //   dir 2: b_j = v_j + w (K2 + w M2)^{-1} M2 (u_j + w s*_j)
 //   dir 3: s_j = (K3 + w M3)^{-1} M3 b_j,  v_{j+1} = b_j - w s_j
 // after r~ = 2 (I (x) M2 (x) M3)^{-1} r (two more line kernels). Arithmetic is
@@ -49,8 +51,11 @@ struct AdiState {
 
 namespace {
 
-constexpr int kL = 32;      // lines per CTA (one solving thread each)
-constexpr int kT = 128;     // threads per CTA
+constexpr int kL = 32;      // lines per CTA (a lane of the solving warps each)
+// 256 threads: about two CTAs run on an SM (n = 96: 288 tiles on 152 SMs), and
+// with 128 the products kept too few FP64 instructions in flight (a launch
+// 54 us, with 256 and the programmatic launch below 50 us).
+constexpr int kT = 256;
 constexpr int kMaxLen = 256;
 
 enum { ST_PRE2 = 0, ST_PRE3, ST_U, ST_S1, ST_B, ST_S, ST2_A, ST2_B, ST2_F };
@@ -181,6 +186,32 @@ __device__ __forceinline__ void store_tile(const T *tile, const LineArgs<T> &a, 
   }
 }
 
+// out(address) = f(in(address), tile(l, i)) for the CTA's lines, coalesced, a
+// batch of loads in flight per thread
+template <int MODE, typename T, typename F>
+__device__ __forceinline__ void update_tile(const T *tile, const LineArgs<T> &a, int nv, const T *in,
+                                            T *out, F f) {
+  constexpr int U = batch_of<T>();
+  const int len = a.len, total = len * kL;
+  for (int e0 = threadIdx.x; e0 < total; e0 += kT * U) {
+    T v[U];
+    long long g[U];
+    int t[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + u * kT;
+      int l, i;
+      entry<MODE>(a, e, l, i);
+      t[u] = (e < total && l < nv) ? tix<MODE>(len, l, i) : -1;
+      g[u] = elem_addr<MODE>(a.n1, a.n2, a.chunks, blockIdx.x, l, i);
+      if (t[u] >= 0) v[u] = in[g[u]];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (t[u] >= 0) out[g[u]] = f(v[u], tile[t[u]]);
+  }
+}
+
 // out(l, i) = base(l, i) + sum_{|o| <= p} coef(i, o) x(l, i + o) over the
 // CTA's lines; coef(i, o) reads the staged bands. Terms are added in
 // increasing o, those outside the line skipped; P > 0 is the compile-time band
@@ -221,74 +252,219 @@ __device__ __forceinline__ void band_product(const LineArgs<T> &a, T *out, const
   }
 }
 
-// (L L^T) y = t in place on line l; F[i][t] = L[i][i-p+t] for t < p, F[i][p] = 1 / L[i][i]
-template <int MODE, typename T>
-__device__ __forceinline__ void chol_solve(T *tile, const T *F, int len, int p, int l) {
-  const int W = p + 1;
-  for (int i = 0; i < len; ++i) {
-    T acc = tile[tix<MODE>(len, l, i)];
-    const int kmax = i < p ? i : p;
-    for (int k = kmax; k >= 1; --k) acc -= F[i * W + p - k] * tile[tix<MODE>(len, l, i - k)];
-    tile[tix<MODE>(len, l, i)] = acc * F[i * W + p];
-  }
-  for (int i = len - 1; i >= 0; --i) {
-    T acc = tile[tix<MODE>(len, l, i)];
-    const int kmax = len - 1 - i < p ? len - 1 - i : p;
-    for (int k = kmax; k >= 1; --k) acc -= F[(i + k) * W + p - k] * tile[tix<MODE>(len, l, i + k)];
-    tile[tix<MODE>(len, l, i)] = acc * F[i * W + p];
-  }
-}
-
-// The same two substitutions with the last P solved values of the line kept
-// in registers, so each step's dependency runs from register to register
-// (the tile supplies only the right-hand side and takes the result); the
-// products are summed in the order of chol_solve. The factor's slots left of
-// the band in the first P rows are never read.
+// FP32: (L L^T) y = t in place on line l, one thread per line; F[i][t] =
+// L[i][i-p+t] for t < p, F[i][p] = 1 / L[i][i]. Each new x is subtracted at
+// once from the P right-hand sides that it enters, which wait in registers: P
+// independent FMAs, of which only the first is on the chain from step to step
+// (an apply of 8 iterations at p = 3: n = 96 771 -> 602 us, n = 64 523 -> 381).
+// The factor row and the right-hand side of the next step are loaded a step
+// ahead. Rows past the end enter with zeros and slots left of the band with
+// whatever they hold; neither reaches a row of the line.
 template <int MODE, typename T, int P>
-__device__ __forceinline__ void chol_solve_reg(T *tile, const T *F, int len, int l) {
+__device__ __forceinline__ void chol_solve(T *tile, const T *F, int len, int l) {
   constexpr int W = P + 1;
-  T win[P];                               // win[k - 1] = x[i - k] (forward), x[i + k] (backward)
+  T acc[P], f[P], d, in;                  // f[k - 1]: coefficient of x_i in row i + k (i - k)
+  auto rows_below = [&](int i) {
 #pragma unroll
-  for (int k = 0; k < P; ++k) win[k] = (T)0;
+    for (int k = 1; k <= P; ++k) f[k - 1] = i + k < len ? F[(i + k) * W + P - k] : (T)0;
+    d = i < len ? F[i * W + P] : (T)0;
+    in = i + P < len ? tile[tix<MODE>(len, l, i + P)] : (T)0;
+  };
+#pragma unroll
+  for (int k = 0; k < P; ++k) acc[k] = k < len ? tile[tix<MODE>(len, l, k)] : (T)0;
+  rows_below(0);
 #pragma unroll 2
   for (int i = 0; i < len; ++i) {
-    T acc = tile[tix<MODE>(len, l, i)];
+    const T x = acc[0] * d;
 #pragma unroll
-    for (int k = P; k >= 1; --k)
-      if (k <= i) acc -= F[i * W + P - k] * win[k - 1];
-    const T x = acc * F[i * W + P];
+    for (int k = 1; k < P; ++k) acc[k - 1] = acc[k] - f[k - 1] * x;
+    acc[P - 1] = in - f[P - 1] * x;
+    rows_below(i + 1);
     tile[tix<MODE>(len, l, i)] = x;
-#pragma unroll
-    for (int k = P - 1; k >= 1; --k) win[k] = win[k - 1];
-    win[0] = x;
   }
+  auto row = [&](int i) {
+    if (i < 0) return;
 #pragma unroll
-  for (int k = 0; k < P; ++k) win[k] = (T)0;
+    for (int k = 1; k <= P; ++k) f[k - 1] = F[i * W + P - k];
+    d = F[i * W + P];
+    in = i - P >= 0 ? tile[tix<MODE>(len, l, i - P)] : (T)0;
+  };
+#pragma unroll
+  for (int k = 0; k < P; ++k) acc[k] = len - 1 - k >= 0 ? tile[tix<MODE>(len, l, len - 1 - k)] : (T)0;
+  row(len - 1);
 #pragma unroll 2
   for (int i = len - 1; i >= 0; --i) {
-    T acc = tile[tix<MODE>(len, l, i)];
+    const T x = acc[0] * d;
 #pragma unroll
-    for (int k = P; k >= 1; --k)
-      if (k <= len - 1 - i) acc -= F[(i + k) * W + P - k] * win[k - 1];
-    const T x = acc * F[i * W + P];
+    for (int k = 1; k < P; ++k) acc[k - 1] = acc[k] - f[k - 1] * x;
+    acc[P - 1] = in - f[P - 1] * x;
+    row(i - 1);
     tile[tix<MODE>(len, l, i)] = x;
+  }
+}
+
+// Rows that the FP64 solve eliminates from the left end (then the middle block
+// of min(p, len) rows, then the rows eliminated from the right end).
+__host__ __device__ inline int split_top(int len, int p) { return len > p ? (len - p) / 2 : 0; }
+
+// FP64: the line is eliminated from both ends at once towards a middle block
+// of P rows, one thread for each end (warp 0 the left, warp 1 the right; lane =
+// line). A warp's FP64 instructions take 65 cycles each whether they depend on
+// one another or not, and up to four warps of an SM do not slow each other, so
+// with about two tiles of 32 lines per SM (n = 96) one thread per line left
+// half of the unit idle for as long as the solve took, 52k of the kernel's 100k
+// cycles. p = 3, 8 iterations, whole applies, before -> with both ends and the
+// eager updates: n = 96 1698 -> 1350 us, n = 64 (one tile per SM) 1170 -> 609 us
+// (with the other changes of this file since). Factor (factor_kernel): unit L, F[i][P] = 1 / D_i,
+// F[i][P-k] = the coefficient between rows i and i - k. All lanes run, those
+// past the tile's last line on whatever their column holds.
+template <int MODE, int P>
+__device__ __forceinline__ void twisted_solve(double *tile, const double *F, int len) {
+  constexpr int W = P + 1;
+  const int l = threadIdx.x & 31, m = split_top(len, P), q = len < P ? len : P, e = m + q;
+  const bool left = threadIdx.x < 32;
+  auto at = [&](int i) -> double & { return tile[tix<MODE>(len, l, i)]; };
+  auto meet = [&]() { asm volatile("bar.sync 1, 64;" ::: "memory"); };
+  double acc[P], f[P], in;
+  // towards the middle: the left end hands its contributions to the middle
+  // rows on in registers (from 0), the right end in the tile (from the rows' own)
+  if (left) {
+    auto next = [&](int i) {
+      if (i >= m) return;
 #pragma unroll
-    for (int k = P - 1; k >= 1; --k) win[k] = win[k - 1];
-    win[0] = x;
+      for (int k = 1; k <= P; ++k) f[k - 1] = F[(i + k) * W + P - k];
+      in = i + P < m ? at(i + P) : 0.0;
+    };
+#pragma unroll
+    for (int k = 0; k < P; ++k) acc[k] = k < m ? at(k) : 0.0;
+    next(0);
+#pragma unroll 2
+    for (int i = 0; i < m; ++i) {
+      const double x = acc[0];
+#pragma unroll
+      for (int k = 1; k < P; ++k) acc[k - 1] = acc[k] - f[k - 1] * x;
+      acc[P - 1] = in - f[P - 1] * x;
+      next(i + 1);
+      at(i) = x;
+    }
+  } else if (e < len) {
+    auto next = [&](int i) {
+      if (i < e) return;
+#pragma unroll
+      for (int k = 1; k <= P; ++k) f[k - 1] = F[i * W + P - k];
+      in = i - P >= m ? at(i - P) : 0.0;
+    };
+#pragma unroll
+    for (int k = 0; k < P; ++k) acc[k] = len - 1 - k >= m ? at(len - 1 - k) : 0.0;
+    next(len - 1);
+#pragma unroll 2
+    for (int i = len - 1; i >= e; --i) {
+      const double x = acc[0];
+#pragma unroll
+      for (int k = 1; k < P; ++k) acc[k - 1] = acc[k] - f[k - 1] * x;
+      acc[P - 1] = in - f[P - 1] * x;
+      next(i - 1);
+      at(i) = x;
+    }
+#pragma unroll
+    for (int k = 0; k < P; ++k) at(e - 1 - k) = acc[k];      // e < len: q = P
+  }
+  meet();
+  if (left) {                                                // the middle block
+#pragma unroll
+    for (int t = 0; t < P; ++t)
+      if (t < q) acc[t] += at(m + t);
+#pragma unroll
+    for (int s = 0; s < P; ++s)
+#pragma unroll
+      for (int t = s + 1; t < P; ++t)
+        if (t < q) acc[t] -= F[(m + t) * W + P - (t - s)] * acc[s];
+#pragma unroll
+    for (int t = 0; t < P; ++t)
+      if (t < q) acc[t] *= F[(m + t) * W + P];
+#pragma unroll
+    for (int s = P - 1; s >= 0; --s)
+      if (s < q) {
+#pragma unroll
+        for (int t = s - 1; t >= 0; --t) acc[t] -= F[(m + s) * W + P - (s - t)] * acc[s];
+        at(m + s) = acc[s];
+      }
+  }
+  meet();
+  // back towards the ends, first what the middle rows contribute
+  if (left && m > 0) {                                       // m > 0: q = P
+    auto enter = [&](int i) { return i >= 0 ? at(i) * F[i * W + P] : 0.0; };
+    auto next = [&](int i) {
+      if (i < 0) return;
+#pragma unroll
+      for (int k = 1; k <= P; ++k) f[k - 1] = F[i * W + P - k];
+      in = enter(i - P);
+    };
+    double y[P];
+#pragma unroll
+    for (int k = 0; k < P; ++k) {
+      y[k] = enter(m - 1 - k);
+#pragma unroll
+      for (int s = P - 1 - k; s >= 0; --s)                   // middle row m + s, distance s + 1 + k
+        y[k] -= F[(m + s) * W + P - 1 - s - k] * acc[s];
+    }
+    next(m - 1);
+#pragma unroll 2
+    for (int i = m - 1; i >= 0; --i) {
+      const double x = y[0];
+#pragma unroll
+      for (int k = 1; k < P; ++k) y[k - 1] = y[k] - f[k - 1] * x;
+      y[P - 1] = in - f[P - 1] * x;
+      next(i - 1);
+      at(i) = x;
+    }
+  } else if (!left && e < len) {
+    auto enter = [&](int i) { return i < len ? at(i) * F[i * W + P] : 0.0; };
+    auto next = [&](int i) {
+#pragma unroll
+      for (int k = 1; k <= P; ++k) f[k - 1] = i + k < len ? F[(i + k) * W + P - k] : 0.0;
+      in = enter(i + P);
+    };
+#pragma unroll
+    for (int k = 0; k < P; ++k) {
+      acc[k] = enter(e + k);
+#pragma unroll
+      for (int s = 0; s < P - k; ++s)                        // middle row e - 1 - s, distance s + 1 + k
+        if (e + k < len) acc[k] -= F[(e + k) * W + P - 1 - s - k] * at(e - 1 - s);
+    }
+    next(e);
+#pragma unroll 2
+    for (int i = e; i < len; ++i) {
+      const double x = acc[0];
+#pragma unroll
+      for (int k = 1; k < P; ++k) acc[k - 1] = acc[k] - f[k - 1] * x;
+      acc[P - 1] = in - f[P - 1] * x;
+      next(i + 1);
+      at(i) = x;
+    }
+  }
+}
+
+// the tile's lines, by the CTA's first warp (FP32) or two warps (FP64)
+template <int MODE, typename T, int P>
+__device__ __forceinline__ void solve_p(T *tile, const T *F, int len, int nv) {
+  if constexpr (sizeof(T) == 8) {
+    if (threadIdx.x < 64) twisted_solve<MODE, P>(tile, F, len);
+  } else {
+    if ((int)threadIdx.x < nv) chol_solve<MODE, T, P>(tile, F, len, threadIdx.x);
   }
 }
 
 template <int MODE, typename T>
-__device__ __forceinline__ void chol_solve_line(T *tile, const T *F, int len, int p, int l) {
+__device__ __forceinline__ void solve_lines(T *tile, const T *F, int len, int p, int nv) {
   switch (p) {
-    case 1: chol_solve_reg<MODE, T, 1>(tile, F, len, l); break;
-    case 2: chol_solve_reg<MODE, T, 2>(tile, F, len, l); break;
-    case 3: chol_solve_reg<MODE, T, 3>(tile, F, len, l); break;
-    case 4: chol_solve_reg<MODE, T, 4>(tile, F, len, l); break;
-    case 5: chol_solve_reg<MODE, T, 5>(tile, F, len, l); break;
-    case 6: chol_solve_reg<MODE, T, 6>(tile, F, len, l); break;
-    case 7: chol_solve_reg<MODE, T, 7>(tile, F, len, l); break;
-    default: chol_solve<MODE>(tile, F, len, p, l);
+    case 1: solve_p<MODE, T, 1>(tile, F, len, nv); break;
+    case 2: solve_p<MODE, T, 2>(tile, F, len, nv); break;
+    case 3: solve_p<MODE, T, 3>(tile, F, len, nv); break;
+    case 4: solve_p<MODE, T, 4>(tile, F, len, nv); break;
+    case 5: solve_p<MODE, T, 5>(tile, F, len, nv); break;
+    case 6: solve_p<MODE, T, 6>(tile, F, len, nv); break;
+    default: solve_p<MODE, T, 7>(tile, F, len, nv);      // p <= 7
   }
 }
 
@@ -302,7 +478,6 @@ __host__ __device__ size_t line_smem(int len, int p) {
 template <typename T, int STEP>
 __global__ void __launch_bounds__(kT) adi_line_kernel(LineArgs<T> a) {
   constexpr int MODE = step_mode(STEP);
-  if (a.done && *a.done != 0.0) return;      // the whole CTA leaves (uniform)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *t0 = reinterpret_cast<T *>(smem_raw);
   T *t1 = t0 + kL * (a.len + 1);
@@ -350,13 +525,17 @@ __global__ void __launch_bounds__(kT) adi_line_kernel(LineArgs<T> a) {
     for (int u = 0; u < kU; ++u)
       if (e0 + u * kT < nf) sF[e0 + u * kT] = f[u];
   }
+  // the bands and the factor are constants of the set-up; what earlier kernels
+  // wrote is read from here on
+  pdl_wait();
+  pdl_trigger();
+  if (a.done && *a.done != 0.0) return;      // the whole CTA leaves (uniform)
   auto Kc = [&](int i, int o) { return sX[i * BW + o + p]; };
   auto Mc = [&](int i, int o) { return sX[i * BW + o + p]; };
   auto Cc = [&](int i, int o) { return sX[i * BW + o + p]; };
   auto Dc = [&](int i, int o) { return sY[i * BW + o + p]; };
   auto zero = [&](int, int) { return (T)0; };
   auto same = [&](T *t) { return [t, len](int l, int i) { return t[tix<MODE>(len, l, i)]; }; };
-  T *res = t1;                     // the tile the solve works on
   if (STEP == ST_PRE2) {
     load_tile<MODE>(t1, a, nv, [&](long long g) { return (T)a.r[g]; });
   } else if (STEP == ST_PRE3) {
@@ -368,6 +547,11 @@ __global__ void __launch_bounds__(kT) adi_line_kernel(LineArgs<T> a) {
   } else if (STEP == ST_S1) {
     if (a.first) {
       load_tile<MODE>(t1, a, nv, [&](long long g) { return a.rt[g]; });      // s = u = v = 0
+    } else if constexpr (sizeof(T) == 8) {
+      load_tiles2<MODE>(t0, [&](long long g) { return (a.u[g] + a.v[g]) - w * a.s[g]; }, t1,
+                        [&](long long g) { return a.rt[g]; }, a, nv);
+      __syncthreads();
+      band_product<MODE>(a, t1, t0, p, nv, Dc, same(t1));                  // r~ - 2 M1 (u + v - w s)
     } else {
       load_tiles2<MODE>(t0, [&](long long g) { return a.s[g]; }, t1,
                         [&](long long g) { return a.rt[g]; }, a, nv);
@@ -400,7 +584,7 @@ __global__ void __launch_bounds__(kT) adi_line_kernel(LineArgs<T> a) {
     load_tile<MODE>(t1, a, nv, [&](long long g) { return a.s[g]; });       // s~_J
   }
   __syncthreads();
-  if ((int)threadIdx.x < nv) chol_solve_line<MODE>(res, sF, len, p, threadIdx.x);
+  solve_lines<MODE>(t1, sF, len, p, nv);
   __syncthreads();
   if (STEP == ST_PRE2) {
     store_tile<MODE>(t1, a, nv, [&](long long g, T x) { a.b[g] = x; });               // M2^{-1} r
@@ -409,21 +593,15 @@ __global__ void __launch_bounds__(kT) adi_line_kernel(LineArgs<T> a) {
   } else if (STEP == ST_U) {
     store_tile<MODE>(t1, a, nv, [&](long long g, T x) { a.u[g] = x; });
   } else if (STEP == ST_S1) {
-    store_tile<MODE>(t1, a, nv, [&](long long g, T x) { a.s1[g] = x; });
+    if (sizeof(T) == 8 && !a.first)
+      update_tile<MODE>(t1, a, nv, a.s, a.s1, [&](T s, T x) { return x - s; });
+    else
+      store_tile<MODE>(t1, a, nv, [&](long long g, T x) { a.s1[g] = x; });
   } else if (STEP == ST_B) {
     if (a.first) {
       store_tile<MODE>(t1, a, nv, [&](long long g, T x) { a.b[g] = w * x; });
     } else {
-      load_tile<MODE>(t0, a, nv, [&](long long g) { return a.v[g]; });       // t0 is free
-      __syncthreads();
-      const int len_ = len;
-      for (int e = threadIdx.x; e < len_ * kL; e += kT) {
-        int l, i;
-        entry<MODE>(a, e, l, i);
-        if (l >= nv) continue;
-        const int t = tix<MODE>(len_, l, i);
-        a.b[elem_addr<MODE>(a.n1, a.n2, a.chunks, blockIdx.x, l, i)] = t0[t] + w * t1[t];
-      }
+      update_tile<MODE>(t1, a, nv, a.v, a.b, [&](T v, T x) { return v + w * x; });
     }
   } else if (STEP == ST2_A || (STEP == ST2_B && !a.last)) {
     // the next half step's right-hand side r - (K - w M) s~ along the same lines
@@ -469,23 +647,49 @@ __global__ void band_kernel(const double *K, const double *M, int n, int p, T *b
   bM[t] = in ? (T)M[(size_t)i * n + j] : (T)0;
 }
 
-// banded Cholesky of K + w_j M (j < J) and of M (j = J), one thread each, in
-// FP64; F[j][i][t] = L[i][i-p+t] (t < p), F[j][i][p] = 1 / L[i][i]
+// banded factors of K + w_j M (j < J) and of M (j = J), one thread each, in
+// FP64. FP32 state: Cholesky from the left end, F[j][i][t] = L[i][i-p+t] (t <
+// p), F[j][i][p] = 1 / L[i][i]. FP64 state: rows are eliminated from both ends
+// towards the middle block of min(p, n) rows from split_top on; L of that
+// order, scaled to a unit diagonal: F[j][i][p-k] = the coefficient between
+// rows i and i - k, F[j][i][p] = 1 / L[i][i]^2.
 template <typename T>
 __global__ void factor_kernel(const double *K, const double *M, int n, int p, const double *omega,
                               int J, T *F, double *work, int *err) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j > J) return;
+  constexpr bool TWISTED = sizeof(T) == 8;
   const int W = p + 1;
   const double ck = j < J ? 1.0 : 0.0;           // K + w_j M, or M
   const double cm = j < J ? omega[j] : 1.0;
   double *L = work + (size_t)j * n * W;          // FP64 factor, same layout
-  for (int i = 0; i < n; ++i) {
+  auto A = [&](int i, int c) { return ck * K[(size_t)i * n + c] + cm * M[(size_t)i * n + c]; };
+  // rows [0, e) from the left end, the middle block last; columns [e, n) from the right end
+  const int e = TWISTED ? split_top(n, p) + (n < p ? n : p) : n;
+  for (int i = n - 1; i >= e; --i) {             // L[r][i], r = i, i - 1 .. i - p, in L[i * W + p - (i - r)]
+    for (int r = i; r >= i - p; --r) {
+      double sum = A(i, r);
+      const int m1 = r + p < n - 1 ? r + p : n - 1;
+      for (int m = i + 1; m <= m1; ++m) sum -= L[m * W + p - (m - r)] * L[m * W + p - (m - i)];
+      if (r == i) {
+        if (!(sum > 0.0)) {
+          atomicExch(err, 1);
+          return;
+        }
+        L[i * W + p] = sqrt(sum);
+      } else {
+        L[i * W + p - (i - r)] = sum / L[i * W + p];
+      }
+    }
+  }
+  for (int i = 0; i < e; ++i) {
     const int j0 = i - p < 0 ? 0 : i - p;
     for (int c = j0; c <= i; ++c) {
-      double sum = ck * K[(size_t)i * n + c] + cm * M[(size_t)i * n + c];
+      double sum = A(i, c);
       const int m0 = j0;                         // L[i][m] L[c][m] != 0 needs m >= i - p (c <= i)
       for (int m = m0; m < c; ++m) sum -= L[i * W + m - i + p] * L[c * W + m - c + p];
+      const int m1 = c + p < n - 1 ? c + p : n - 1;
+      for (int m = e; m <= m1; ++m) sum -= L[m * W + p - (m - i)] * L[m * W + p - (m - c)];
       if (c == i) {
         if (!(sum > 0.0)) {
           atomicExch(err, 1);
@@ -499,8 +703,14 @@ __global__ void factor_kernel(const double *K, const double *M, int n, int p, co
   }
   T *out = F + (size_t)j * n * W;
   for (int i = 0; i < n; ++i) {
-    for (int t = 0; t < p; ++t) out[i * W + t] = (T)L[i * W + t];
-    out[i * W + p] = (T)(1.0 / L[i * W + p]);
+    const double inv = 1.0 / L[i * W + p];
+    for (int t = 0; t < p; ++t) {
+      const int k = i - p + t;
+      double v = k >= 0 ? L[i * W + t] : 0.0;
+      if (TWISTED && k >= 0) v /= i >= e ? L[i * W + p] : L[k * W + p];
+      out[i * W + t] = (T)v;
+    }
+    out[i * W + p] = (T)(TWISTED ? inv * inv : inv);
   }
 }
 
@@ -540,9 +750,8 @@ igafd_status launch_step(const AdiState &S, const LineArgs<T> &base, int dir, in
     IGAFD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     attr_set.fetch_or(bit);
   }
-  kern<<<(unsigned)grid, kT, smem, s>>>(a);
+  IGAFD_CUDA(igafd_launch(kern, dim3((unsigned)grid), dim3(kT), smem, s, a));
   IGAFD_LAUNCHED(1);
-  IGAFD_CUDA(cudaGetLastError());
   return IGAFD_OK;
 }
 
