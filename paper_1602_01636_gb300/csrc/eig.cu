@@ -986,7 +986,9 @@ struct GemmBatch {
 
 // 8 x 8 output tile per CTA (64 threads), K in panels of 64: at n = 128 a
 // product is 256 CTAs, spread over all SMs (one SM's FP64 rate is low, so
-// the products want as many SMs as possible).
+// the products want as many SMs as possible). A panel's sixteen loads per
+// thread are all issued before the first is stored (one after another they
+// took longer than the FMAs: a 2D solve at n = 64 736 -> 727 us, nine products).
 constexpr int kGT = 8;
 __global__ void __launch_bounds__(64) gemm64_kernel(GemmBatch b) {
   const GemmJob g = b.j[blockIdx.y];
@@ -1009,16 +1011,20 @@ __global__ void __launch_bounds__(64) gemm64_kernel(GemmBatch b) {
   const int row = ti * kGT + ty, col = tj * kGT + tx;
   double acc = 0.0;
   for (int k0 = 0; k0 < n; k0 += KP) {
-    for (int t = threadIdx.x; t < kGT * KP; t += kGT * kGT) {
-      if (g.transA) {
-        const int kk = t / kGT, r = t % kGT, ra = ti * kGT + r, ka = k0 + kk;
-        As[r][kk] = (ra < n && ka < n) ? g.A[(size_t)ka * n + ra] : 0.0;
-      } else {
-        const int r = t / KP, kk = t % KP, ra = ti * kGT + r, ka = k0 + kk;
-        As[r][kk] = (ra < n && ka < n) ? g.A[(size_t)ra * n + ka] : 0.0;
-      }
-      const int kk = t / kGT, c = t % kGT, kb = k0 + kk, cb = tj * kGT + c;
-      Bs[kk][c] = (kb < n && cb < n) ? g.B[(size_t)kb * n + cb] : 0.0;
+    double av[KP / kGT], bv[KP / kGT];
+#pragma unroll
+    for (int u = 0; u < KP / kGT; ++u) {
+      const int t = threadIdx.x + u * kGT * kGT, kt = t / kGT, ct = t % kGT;
+      const int ra = ti * kGT + (g.transA ? ct : t / KP), ka = k0 + (g.transA ? kt : t % KP);
+      const int cb = tj * kGT + ct, kb = k0 + kt;
+      av[u] = (ra < n && ka < n) ? g.A[g.transA ? (size_t)ka * n + ra : (size_t)ra * n + ka] : 0.0;
+      bv[u] = (kb < n && cb < n) ? g.B[(size_t)kb * n + cb] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < KP / kGT; ++u) {
+      const int t = threadIdx.x + u * kGT * kGT, kt = t / kGT, ct = t % kGT;
+      As[g.transA ? ct : t / KP][g.transA ? kt : t % KP] = av[u];
+      Bs[kt][ct] = bv[u];
     }
     __syncthreads();
 #pragma unroll 16
