@@ -398,13 +398,12 @@ igafd_status igafd_apply_prec_static(int dim, const int *n, const double *const 
 igafd_status igafd_setup_prec(igafd_patch *patch, void *stream);
 
 /* Eigen-solver route for the next setup of P: 0 (default) = for every
- * direction, an FP32 start (Householder tridiagonalisation, bisection,
- * inverse iteration; in shared memory for n_k <= 128) followed by FP64
+ * direction with n_k <= 128 or p <= 2, an FP32 start (Householder
+ * tridiagonalisation, bisection, inverse iteration) followed by FP64
  * iterative refinement of the eigenvectors (Ogita and Aishima, 2018) and
  * exact rotations of nearly degenerate pairs, accepted only if
  * max |U~^T U~ - I| <= 1e-12 and the off-diagonal of U~^T K~ U~ is <= 1e-12
- * of its diagonal, else FP64 cyclic Jacobi; 1 = FP64
- * Jacobi for every direction. igafd_patch_info.eig_refined reports the
+ * of its diagonal; FP64 cyclic Jacobi otherwise; 1 = FP64 Jacobi for every direction. igafd_patch_info.eig_refined reports the
  * route each direction took. Other values: IGAFD_ERR_ARG. */
 igafd_status igafd_set_eig_route(igafd_patch *patch, int route);
 

@@ -622,10 +622,20 @@ __global__ void __launch_bounds__(1024) tri32_kernel(EigJob *jobs, int allow_fas
 // once). Every pass over a matrix walks its rows, coalesced; L1 holds much of
 // it up to n of about 200. One CTA does the start up to T's eigenvectors;
 // back32_kernel takes them back to the pencil's, columns spread over CTAs.
-// Measured, the whole eigendecomposition with the refinement: 1.5 ms at n =
-// 150, 2.1 at 192, 6 at 300, 24 at 512, where FP64 Jacobi took 73, 161, 647 and
-// 3600 ms. Bound by the tridiagonalisation's passes over the matrix (one CTA).
+// Measured at p = 3 before the degree limit below (the work hardly depends on
+// p), the whole eigendecomposition with the refinement: 1.5 ms at n = 150,
+// 2.1 at 192, 6 at 300, 24 at 512, where FP64 Jacobi took 73, 161, 647 and 3600 ms. Bound by the tridiagonalisation's passes over the matrix (one CTA).
 constexpr int kBigMaxN = 1024;
+
+// Degrees up to which the route takes n > kFastMaxN. From p = 3 on, pencils on
+// uniform knots have pairs of outlier eigenvalues (one function at either end)
+// that agree to rounding: any basis of such a pair is an eigenbasis, and an
+// FD with rounded operands gives another rounding for another basis (TF32
+// applies at (150, 140, 60), p = 3: 3e-4 between the two, each 7e-4 from FP64).
+// Those keep the FP64 Jacobi's basis. At p <= 2 the eigenvalues are apart, and
+// the applies of either route are equal bit for bit in TF32, BF16, FP16 and
+// FP32 ((160, 37, 129), p = 2).
+constexpr int kBigMaxP = 2;
 
 // eight threads per eigenvalue: 9-way multisection on Sturm counts (the
 // interval shrinks by 9 per round)
@@ -684,7 +694,7 @@ __host__ __device__ constexpr size_t big32_smem_floats(int n) { return (size_t)n
 __global__ void __launch_bounds__(1024) big32_kernel(EigJob *jobs, int allow_fast) {
   EigJob jb = jobs[blockIdx.x];
   const int n = jb.n, p = jb.p;
-  if (!allow_fast || n <= kFastMaxN || p >= kMaxBand) return;   // tri32_kernel's pencils
+  if (!allow_fast || n <= kFastMaxN || p > kBigMaxP) return;   // tri32_kernel's pencils, or Jacobi's
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt / 32;
   extern __shared__ float t32[];
   float *vv = t32, *pw = vv + n, *dd = pw + n, *ee = dd + n, *e2 = ee + n, *bet = e2 + n, *lam = bet + n;
@@ -1527,8 +1537,8 @@ igafd_status igafd_setup_pencils_eig(igafd_patch *P, cudaStream_t s, const doubl
     const int k = dir_of[u];
     int n = P->n[k];
     max_n = n > max_n ? n : max_n;
-    fast_jobs += p < kMaxBand;
-    big_jobs += n > kFastMaxN;
+    fast_jobs += n <= kFastMaxN ? p < kMaxBand : p <= kBigMaxP;
+    big_jobs += n > kFastMaxN && p <= kBigMaxP;
     size_t nn = (size_t)n * n;
     EigJob &j = hjobs[u];
     double *w = P->eig_work + off;
