@@ -45,7 +45,7 @@ struct AdiState {
   size_t esz = 8;                  // bytes per element (8 FP64, 4 FP32)
   double *omega = nullptr;         // [J] host copy
   void *band[3] = {nullptr, nullptr, nullptr};   // [2][n][2p+1]: K band, M band
-  void *fac[3] = {nullptr, nullptr, nullptr};    // [J+1][n][p+1]: K + w_j M (j < J), M (j = J)
+  void *fac[3] = {nullptr, nullptr, nullptr};    // [J+1][n][p+1]: K + w_j M (j < J), M (j = J); see factor_kernel
   void *vec = nullptr;             // 6 N-vectors: r~, u, v, s, s*, b
 };
 
@@ -76,7 +76,7 @@ struct LineArgs {
   double *z;                       // FP64 output (ST_S of the last iteration)
   T *rt, *u, *v, *s, *s1, *b;      // N-vectors
   const T *bK, *bM;                // bands of this direction's pencil [n][2p+1]
-  const T *fac;                    // Cholesky factor used by the solve [n][p+1]
+  const T *fac;                    // factor used by the solve [n][p+1]
   const double *done;              // PCG convergence flag: skip all work while != 0 (or null)
 };
 

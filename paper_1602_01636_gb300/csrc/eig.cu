@@ -624,7 +624,8 @@ __global__ void __launch_bounds__(1024) tri32_kernel(EigJob *jobs, int allow_fas
 // back32_kernel takes them back to the pencil's, columns spread over CTAs.
 // Measured at p = 3 before the degree limit below (the work hardly depends on
 // p), the whole eigendecomposition with the refinement: 1.5 ms at n = 150,
-// 2.1 at 192, 6 at 300, 24 at 512, where FP64 Jacobi took 73, 161, 647 and 3600 ms. Bound by the tridiagonalisation's passes over the matrix (one CTA).
+// 2.1 at 192, 6 at 300, 24 at 512, where FP64 Jacobi took 73, 161, 647 and 3600
+// ms. Bound by the tridiagonalisation's passes over the matrix (one CTA).
 constexpr int kBigMaxN = 1024;
 
 // Degrees up to which the route takes n > kFastMaxN. From p = 3 on, pencils on
