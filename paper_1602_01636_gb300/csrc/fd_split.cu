@@ -15,7 +15,7 @@
 // with ea_m the largest exponent field of row m and eb_j that of row j of B
 // (U_k^T or U_k, split at set-up). Digits are exact in FP16; the FP32
 // accumulators of tcgen05.mma hold the leading groups' integers exactly (see
-// Steps). Groups g <= 5 are kept (21 digit products); their accumulators
+// Steps in split_plan.h). Groups g <= 5 are kept (21 digit products); their accumulators
 // are summed as 64-bit integers and rounded to FP64 once. In units of 2^-53
 // of the result's norm, a product's error is 0.4-1.8 (0.4 unless one factor's
 // entries decay along the sum) where the FP64 FMA chain of the SIMT kernel
@@ -44,6 +44,7 @@
 // warp-private transposition. The divide's table inv_lam is stored in the
 // layout the third product writes, [j1][j3][j2].
 #include "common.cuh"
+#include "split_plan.h"
 
 #include <atomic>
 #include <cstdlib>
@@ -53,10 +54,11 @@
 
 namespace {
 
+using namespace igafd_split;
+
 constexpr int kM = 128;                 // rows per CTA (MMA M, TMEM lanes)
 constexpr int kThreads = 512;           // 4 warps per lane quarter
 constexpr int kWarps = kThreads / 32;
-constexpr int kSlices = 6;              // digits per operand
 constexpr long long kSpin = 1ll << 26;  // bounded waits
 // X + kBias = sum_s (digit_s + 512) 1024^(5-s): every 10-bit field is then the
 // digit plus 512
@@ -76,24 +78,6 @@ struct SplitArgs {
   const double *inv_lam;      // divide table, indexed like out (null: none)
   const double *done;
   int *err;
-};
-
-// The accumulation steps of a column block for K <= 64 and K <= 128: the
-// group, and its 64-wide K chunks c0 <= c < c1. FP32 accumulation of integers
-// is exact below 2^24, and the chunks keep the sums of the leading groups
-// there: |a_0 b_0| <= 2^17 over 128 terms; the products of groups 1 and 2 have
-// |a| <= 2^9 and, over U_k's entries, |b| of half its 2^9 on average, so their
-// sums over 64 terms stay below 2^23 per product (2^22 with a_0). Group 3
-// weighs 2^-30 of group 0: a rounding there is below the result's last bit.
-struct Step { int g, c0, c1; };
-template <int KP> struct Steps {
-  static constexpr int kCount = KP > 64 ? 8 : 6;
-  __host__ __device__ static constexpr Step at(int i) {
-    if (KP <= 64) return Step{i, 0, 1};
-    if (i == 0) return Step{0, 0, 2};
-    if (i < 5) return Step{(i + 1) / 2, (i - 1) % 2, (i - 1) % 2 + 1};
-    return Step{i - 2, 0, 2};
-  }
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -225,16 +209,10 @@ __device__ __forceinline__ double round_fixed(long long T, int E, double lam, bo
 // columns and half the shared memory each), so one's MMAs and the start of the
 // next launch overlap the other's integer work.
 constexpr int acc_cols(int KP) { return KP > 64 ? 64 : 32; }
-// With K > 128 the rows are split and multiplied in two parts (the first 128
-// terms, then the rest, on the same row exponents) whose groups add up in the
-// 64-bit sums; a CTA then takes at most 64 columns, so that B's digits of both
+// With K > 128 a CTA takes at most 64 columns, so that B's digits of both
 // parts fit.
-constexpr int part_terms(int KP) { return KP > 128 ? 128 : KP; }
 constexpr int b_rows(int KP) { return KP > 128 ? 64 : kM; }
 constexpr int ctas_per_sm(int KP) { return KP > 64 ? 1 : 2; }
-// slices of B fetched before the input is read (the rest of B's shared memory
-// holds the transposition buffers until then)
-constexpr int first_slices(int KP) { return KP > 128 ? kSlices : KP > 64 ? 3 : 1; }
 // doubles per row of a transposition buffer, and its bytes for all warps
 constexpr int trans_cols(int KP) { return KP > 128 ? 8 : 17; }
 constexpr int trans_bytes(int KP) { return 16 * 32 * trans_cols(KP) * 8; }
@@ -440,8 +418,11 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     constexpr int KT = part_ ? KR : KA, KS = KT / 16, kc0 = part_ ? KA / 64 : 0;
     constexpr Step p = Steps<KT>::at(i);
     const int buf = st & 1;
-    if (i == 0 && sub == 0 && part_ == 0) ok = ok && wait_on(&bar_b[0], 0, &s_fail);
-    if (p.g >= kFirst && sub == 0) ok = ok && wait_on(&bar_b[1], 0, &s_fail);
+    if (sub == 0) {                                        // (a poll each once they have arrived)
+      constexpr unsigned waits = step_waits(KP, p.g);
+      if (waits & 1u) ok = ok && wait_on(&bar_b[0], 0, &s_fail);
+      if (waits & 2u) ok = ok && wait_on(&bar_b[1], 0, &s_fail);
+    }
     if (st >= 2) ok = ok && wait_on(&bar_empty[buf], (uint32_t)(((st >> 1) - 1) & 1), &s_fail);
     ok = __all_sync(0xffffffffu, ok);
     if (!ok) return;
