@@ -7,28 +7,31 @@
 // splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012, with
 // integer digits), and the products of digits run on the tensor cores:
 //
-//   a_mi = 2^(ea_m - 1081) sum_s da[s]_mi 1024^(5 - s),   |da[s]| <= 512
-//   b_ji = 2^(eb_j - 1082) sum_t db[t]_ji 1024^(5 - t),   |db[t]| <= 512
-//   sum_i a_mi b_ji = 2^(ea_m + eb_j - 2163) sum_g 1024^(10 - g) G_g,
+//   a_mi = 2^(ea_m - 1080) sum_s da[s]_mi 1024^(5 - s),   |da[0]| <= 256,
+//   b_ji = 2^(eb_j - 1080) sum_t db[t]_ji 1024^(5 - t),   |da[s]| <= 512
+//   sum_i a_mi b_ji = 2^(ea_m + eb_j - 2160) sum_g 1024^(10 - g) G_g,
 //   G_g = sum_{s + t = g} sum_i da[s]_mi db[t]_ji
 //
 // with ea_m the largest exponent field of row m and eb_j that of row j of B
 // (U_k^T or U_k, split at set-up). Digits are exact in FP16; the FP32
-// accumulators of tcgen05.mma hold the leading groups' integers exactly (see
-// Steps in split_plan.h). Groups g <= 5 are kept (21 digit products); their accumulators
-// are summed as 64-bit integers and rounded to FP64 once. In units of 2^-53
-// of the result's norm, a product's error is 0.4-1.8 (0.4 unless one factor's
-// entries decay along the sum) where the FP64 FMA chain of the SIMT kernel
-// has 1.0 (K = 12) to 4.8 (K = 128). The divide by D_1 (+) D_2 (+) D_3
+// accumulators of tcgen05.mma hold the integers of groups 0 to 3 exactly,
+// whatever the digits (split_plan.h). Groups g <= 5 are kept (21 digit
+// products); their accumulators are summed as 64-bit integers and rounded to
+// FP64 once. A product's error is relative to the largest entries of its row
+// and column: in units of 2^-53 of their norms 0.1-0.2 for rows along an
+// eigenvector of degree 1 (an FP64 chain: 6-9), 18 for one large entry among
+// 127 equal ones that are smaller by any factor (chain: 47). The divide by D_1 (+) D_2 (+) D_3
 // multiplies the integer result before that rounding. No FP64 instruction is
 // executed (each would issue at the 2-per-clock rate).
 //
-// Measured: 170 us per apply at n = 128 (SIMT: 3.10 ms), 95 us at (95, 61, 77)
-// (SIMT: 0.98 ms), 1.23 ms at n = 192 (SIMT: 13.8 ms). A pass at n = 128 is bound by integer instructions (64
-// lanes per clock per SM, conversions 16): 20 us, of which reading and
-// splitting the rows 6 us, the MMAs with the summation of their accumulators
-// 9 us (the MMAs alone 5), the last rounding 2.5 us; about 6 us pass between
-// two launches.
+// Measured: 207 us per apply at n = 128 (SIMT: 3.10 ms), 108 us at (95, 61, 77)
+// (SIMT: 0.98 ms). A pass at n = 128 takes the phases of its one tile per SM in
+// turn: reading and splitting the rows (6 us), the MMAs with the summation of
+// their accumulators (the MMAs alone 5 us), the last rounding (2.5 us), and
+// about 6 us between two launches. With groups 1 to 3 in fewer, larger sums
+// (eight instead of fifteen steps at K = 128) an apply took 172 and 94 us, but
+// rows whose digits add up with one sign passed 2^24 and lost up to 3000 units
+// of 2^-53.
 //
 // A CTA takes 128 rows (the other directions' indices) and up to 128 columns.
 // A's digits live in tensor memory (6 slices of K/2 columns: 384 of 512 at
@@ -130,17 +133,15 @@ __device__ __forceinline__ int exp_field(uint32_t hi) {
   return e > 1 ? e : 1;
 }
 
-// X + kBias with X = d 2^(1023 + BITS - ea) truncated, |X| < 2^BITS, as its
-// upper and lower 30 bits (junk above bit 30 of the lower word). A has 58
-// bits, so that its top digit fits the packed conversion; B has 59.
-template <int BITS>
+// X + kBias with X = d 2^(1022 + kBits - ea) rounded down, |X| <= 2^kBits, as
+// its upper and lower 30 bits (junk above bit 30 of the lower word).
 __device__ __forceinline__ void biased_fixed(double d, int ea, uint32_t &w1, uint32_t &w0) {
   const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
   // mantissa with the hidden bit at bit 63 (its place holds the exponent's
   // lowest bit, which is 0 where there is no hidden bit)
   const uint32_t mh = __funnelshift_l(lo, hi, 11) | ((hi & 0x7ff00000u) ? 0x80000000u : 0u);
   const uint32_t ml = lo << 11;
-  const uint32_t sh = (uint32_t)(ea + 64 - BITS - exp_field(hi));
+  const uint32_t sh = (uint32_t)(ea + 64 - kBits - exp_field(hi));
   const uint32_t s1 = min(sh, 32u);
   uint32_t xh = shr_clamp(mh, s1);
   uint32_t xl = shr_clamp(__funnelshift_rc(ml, mh, s1), sh - s1);
@@ -216,6 +217,15 @@ constexpr int ctas_per_sm(int KP) { return KP > 64 ? 1 : 2; }
 // doubles per row of a transposition buffer, and its bytes for all warps
 constexpr int trans_cols(int KP) { return KP > 128 ? 8 : 17; }
 constexpr int trans_bytes(int KP) { return 16 * 32 * trans_cols(KP) * 8; }
+// f(0), f(1), ... f(N - 1), as constants
+template <typename F, int... I>
+__device__ __forceinline__ void each_of(F &&f, std::integer_sequence<int, I...>) {
+  (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, typename F> __device__ __forceinline__ void each_step(F &&f) {
+  each_of(f, std::make_integer_sequence<int, N>{});
+}
+
 template <int KP, bool LAM>
 __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(SplitArgs a) {
   extern __shared__ unsigned char smem_raw[];
@@ -359,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
   auto put_digits = [&](const double (&x)[KQ], int ea) {
     uint32_t w1[KQ], w0[KQ];
 #pragma unroll
-    for (int i = 0; i < KQ; ++i) biased_fixed<58>(x[i], ea, w1[i], w0[i]);
+    for (int i = 0; i < KQ; ++i) biased_fixed(x[i], ea, w1[i], w0[i]);
     auto put = [&](int s, auto pos, const uint32_t *w) {
       constexpr int POS = decltype(pos)::value;
 #pragma unroll
@@ -415,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
   // K terms of part `part` (KT of them, from chunk c0), group and chunks of step i
   auto issue = [&](auto part, auto step, int sub, int st) {   // one warp
     constexpr int i = decltype(step)::value, part_ = decltype(part)::value;
-    constexpr int KT = part_ ? KR : KA, KS = KT / 16, kc0 = part_ ? KA / 64 : 0;
+    constexpr int KT = part_ ? KR : KA, kc0 = part_ ? KA / 64 : 0;
     constexpr Step p = Steps<KT>::at(i);
     const int buf = st & 1;
     if (sub == 0) {                                        // (a poll each once they have arrived)
@@ -437,10 +447,11 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     if (elected) {
 #pragma unroll
       for (int sl = 0; sl <= p.g; ++sl) {
+        if (!(p.prods >> sl & 1u)) continue;
         const uint64_t bs = bsub + (uint32_t)((p.g - sl) * slice_bytes >> 4);
 #pragma unroll
-        for (int ks = 4 * p.c0; ks < KS && ks < 4 * p.c1; ++ks) {
-          const uint32_t acc = sl == 0 && ks == 4 * p.c0 ? 0u : 1u;
+        for (int ks = p.k0; ks < p.k1; ++ks) {
+          const uint32_t acc = (p.prods & ((1u << sl) - 1u)) == 0u && ks == p.k0 ? 0u : 1u;
           asm volatile(
               "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
               " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
@@ -459,7 +470,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
   constexpr int C = kNS / 4;                               // columns per thread in a block
   const bool bad_row = ea == 0x7ff;
   const long long ob = hi * a.out_hi + lo * a.out_lo;
-  constexpr int kTop = KR > 0 ? 37 : 38;                   // weight of group 0 in T
+  constexpr int kTop = KR > 0 ? 38 : 39;                   // weight of group 0 in T
   int st = 0;
   if (warp == 0) issue(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{}, 0, 0);
   for (int sub = 0; sub < nsub; ++sub) {
@@ -498,9 +509,9 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_empty[buf]);
-      // T in units of 2^12 (2^13 with two parts) of group 5: a part's |G_0|
-      // 2^38 <= 2^62; what is dropped of groups 4 and 5 is of the order of the
-      // groups not computed
+      // T in units of 2^11 (2^12 with two parts) of group 5: |G_0| 2^kTop <=
+      // 2^62; what is dropped of groups 4 and 5 is of the order of the groups
+      // not computed
 #pragma unroll
       for (int c = 0; c < C; ++c) {
         const int G = __float2int_rn(__uint_as_float(v[c]));
@@ -511,16 +522,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
       }
     };
     auto sum_part = [&](auto part) {
-      sum(part, std::integral_constant<int, 0>{});
-      sum(part, std::integral_constant<int, 1>{});
-      sum(part, std::integral_constant<int, 2>{});
-      sum(part, std::integral_constant<int, 3>{});
-      sum(part, std::integral_constant<int, 4>{});
-      sum(part, std::integral_constant<int, 5>{});
-      if constexpr (Steps<decltype(part)::value ? KR : KA>::kCount == 8) {
-        sum(part, std::integral_constant<int, 6>{});
-        sum(part, std::integral_constant<int, 7>{});
-      }
+      each_step<Steps<decltype(part)::value ? KR : KA>::kCount>([&](auto step) { sum(part, step); });
     };
     sum_part(std::integral_constant<int, 0>{});
     if constexpr (KR > 0) {                                // (one column block)
@@ -543,7 +545,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     bool slow = bad_row;
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      const double y = round_fixed<LAM>(T[c], ea + (int)s_eb[(nl0 + c) & (kM - 1)] - 2061 - kTop, lam[c], slow);
+      const double y = round_fixed<LAM>(T[c], ea + (int)s_eb[(nl0 + c) & (kM - 1)] - 2060 - kTop, lam[c], slow);
       if (c < ncol) a.out[o0 + c * a.out_n] = y;
     }
     if (slow) {                                          // rare: again, one by one
@@ -552,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
         if (c < ncol)
           a.out[o0 + c * a.out_n] =
               bad_row ? __longlong_as_double(0x7ff8000000000000ll)
-                      : round_slow(T[c], ea + (int)s_eb[nl0 + c] - 2061 - kTop, lam[c]);
+                      : round_slow(T[c], ea + (int)s_eb[nl0 + c] - 2060 - kTop, lam[c]);
     }
   }
   if (!ok) s_fail = 1;
@@ -601,12 +603,12 @@ __global__ void __launch_bounds__(256) split_image_kernel(ImgBatch b) {
   if (k == 0) J.eb[r] = e;
   if (k >= nkc * 64) return;
   uint32_t w1, w0;
-  biased_fixed<59>(d, e, w1, w0);
+  biased_fixed(d, e, w1, w0);
   const int kb = (k & 63) * 2;
   unsigned char *at = J.img + ((size_t)(k >> 6) * J.Np + r) * 128 + ((((kb >> 4) ^ (r & 7)) << 4) | (kb & 15));
   const size_t slice = (size_t)nkc * J.Np * 128;
   auto put = [&](int s, uint32_t w) { *reinterpret_cast<unsigned short *>(at + s * slice) = (unsigned short)w; };
-  put(0, __half_as_ushort(__int2half_rn((int)(w1 >> 20) - 512)));   // -512..512
+  put(0, digit2<2>(w1, w1));
   put(1, digit2<1>(w1, w1));
   put(2, digit2<0>(w1, w1));
   put(3, digit2<2>(w0, w0));

@@ -14,23 +14,61 @@ constexpr int part_terms(int KP) { return KP > 128 ? 128 : KP; }
 // holds the transposition buffers until then)
 constexpr int first_slices(int KP) { return KP > 128 ? kSlices : KP > 64 ? 3 : 1; }
 
-// The accumulation steps of a column block for K <= 64 and K <= 128: the
-// group, and its 64-wide K chunks c0 <= c < c1. FP32 accumulation of integers
-// is exact below 2^24, and the chunks keep the sums of the leading groups
-// there: |a_0 b_0| <= 2^17 over 128 terms; the products of groups 1 and 2 have
-// |a| <= 2^9 and, over U_k's entries, |b| of half its 2^9 on average, so their
-// sums over 64 terms stay below 2^23 per product (2^22 with a_0). Group 3
-// weighs 2^-30 of group 0: a rounding there is below the result's last bit.
-struct Step { int g, c0, c1; };
-template <int KT> struct Steps {
-  static constexpr int kCount = KT > 64 ? 8 : 6;
-  static constexpr Step at(int i) {
-    if (KT <= 64) return Step{i, 0, 1};
-    if (i == 0) return Step{0, 0, 2};
-    if (i < 5) return Step{(i + 1) / 2, (i - 1) % 2, (i - 1) % 2 + 1};
-    return Step{i - 2, 0, 2};
-  }
+// |digit| of either operand: X has 58 bits, so that its top digit is at most
+// 2^8 (with the carry of the digits below), the others lie in -512 .. 511.
+constexpr int kBits = 58;
+constexpr long long digit_bound(int s) { return s == 0 ? 1 << (kBits - 50) : 1 << 9; }
+
+// One accumulation step of a column block: the products a_s b_(g - s) of group
+// g for the bits s of prods, over the 16-term blocks k0 <= k < k1.
+struct Step {
+  int g;
+  unsigned prods;
+  int k0, k1;
 };
+// largest |sum| over `terms` terms
+constexpr long long step_bound(int g, unsigned prods, int terms) {
+  long long b = 0;
+  for (int s = 0; s <= g; ++s)
+    if (prods >> s & 1u) b += digit_bound(s) * digit_bound(g - s);
+  return b * terms;
+}
+
+// The steps for KT <= 128 terms. The FP32 accumulators hold integers exactly up
+// to 2^24, so the sums of groups 0 to 3 are cut where the largest digits could
+// pass it: 64 terms of group 1, 32 of group 2, in group 3 32 of three products
+// and 64 of the fourth. Groups 4 and 5 take all terms at once: their unit is
+// 2^-54 and 2^-64 of the largest a times the largest b, and cutting group 4 at
+// 64 terms changed no error by a tenth of a unit of 2^-53 of the norms.
+constexpr int kExact = 4;
+struct StepList {
+  int n = 0;
+  Step s[16] = {};
+};
+constexpr StepList steps_of(int KT) {
+  StepList l;
+  for (int g = 0; g < kSlices; ++g) {
+    const unsigned all = (2u << g) - 1, sets[2] = {g == 3 ? 0xbu : all, g == 3 ? 0x4u : 0u};
+    for (const unsigned prods : sets) {
+      if (!prods) continue;
+      const int blocks = KT / 16;
+      const int cut = g < kExact ? (int)((1ll << 24) / step_bound(g, prods, 16)) : blocks;
+      for (int k = 0; k < blocks; k += cut) l.s[l.n++] = Step{g, prods, k, k + cut < blocks ? k + cut : blocks};
+    }
+  }
+  return l;
+}
+template <int KT> struct Steps {
+  static constexpr int kCount = steps_of(KT).n;
+  static constexpr Step at(int i) { return steps_of(KT).s[i]; }
+};
+constexpr bool sums_exact(int KT) {
+  const StepList l = steps_of(KT);
+  for (int i = 0; i < l.n; ++i)
+    if (l.s[i].g < kExact && step_bound(l.s[i].g, l.s[i].prods, 16 * (l.s[i].k1 - l.s[i].k0)) > 1ll << 24) return false;
+  return l.s[0].g == 0 && (l.n < 2 || l.s[1].g != 0);    // group 0 in one step
+}
+static_assert(sums_exact(32) && sums_exact(64) && sums_exact(96) && sums_exact(128));
 
 // B's slices arrive by bulk copies on two barriers: slices below first_slices
 // on barrier 0, the others on barrier 1. Bit i: the warp that issues the

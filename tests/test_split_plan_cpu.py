@@ -1,5 +1,7 @@
 """Schedule of the split FP64 FD's digit products (csrc/split_plan.h), as the
-host compiler sees it: every step waits for the slices of B that it reads."""
+host compiler sees it: every step waits for the slices of B that it reads, the
+steps hold every product of the kept groups once, and those of the leading
+groups cannot pass the integers that FP32 accumulates exactly."""
 import os
 import shutil
 import subprocess
@@ -16,7 +18,7 @@ using namespace igafd_split;
 template <int KP, int KT> void steps(int part) {
   for (int i = 0; i < Steps<KT>::kCount; ++i) {
     const Step s = Steps<KT>::at(i);
-    printf("step %d %d %d %d %u\n", KP, part, KT, s.g, step_waits(KP, s.g));
+    printf("step %d %d %d %d %u %d %d %u\n", KP, part, KT, s.g, s.prods, s.k0, s.k1, step_waits(KP, s.g));
   }
 }
 template <int KP> void plan() {
@@ -59,3 +61,18 @@ def test_every_step_waits_for_the_slices_it_reads(plan):
         for g, waits in ((s[0], s[-1]) for s in todo):
             for t in range(g + 1):                     # products of group g read slices 0 .. g of B
                 assert waits >> (0 if t < first[KP] else 1) & 1, (KP, g, t)
+
+
+def test_products_once_and_exact(plan):
+    _, steps, slices = plan
+    big = lambda s: 256 if s == 0 else 512             # 58 bits: 8 above five digits of 10
+    for (_, _, KT), todo in steps.items():
+        seen = []
+        for g, prods, k0, k1, _ in todo:
+            pairs = [(s, g - s) for s in range(slices) if prods >> s & 1]
+            assert pairs and 0 <= k0 < k1 <= KT // 16
+            seen += [(s, t, k) for s, t in pairs for k in range(k0, k1)]
+            if g <= 3:
+                assert 16 * (k1 - k0) * sum(big(s) * big(t) for s, t in pairs) <= 2 ** 24
+        want = [(s, g - s, k) for g in range(slices) for s in range(g + 1) for k in range(KT // 16)]
+        assert sorted(seen) == sorted(want)
