@@ -48,7 +48,15 @@ typedef enum {
 /* Arithmetic of the preconditioner's mode-k contractions. The outer PCG
  * (inner products, residual recurrence, A stencil) is always FP64. */
 typedef enum {
-  IGAFD_FP64 = 0,   /* FP64 contractions and divide: FD is exactly P^{-1} */
+  IGAFD_FP64 = 0,   /* FD is P^{-1} up to FP64 rounding. With every n_k <= 256 each
+                       contraction is formed from 58-bit digits on the tensor
+                       cores and rounded to FP64 once: its error is relative to
+                       the largest entries of the contracted row of the input
+                       and of the row of U_k, not to each product's size.
+                       Directions where the rows of U_k differ by more than
+                       about 2^4 (spans graded by more than about 50, span
+                       scalings of that size), and n_k > 256, take FP64 FMA
+                       chains */
   IGAFD_FP32 = 1,   /* FP32 SIMT contractions, FP32 divide */
   IGAFD_BF16 = 2,   /* tcgen05 kind::f16 with bf16 operands, FP32 accumulate */
   IGAFD_FP16 = 3,   /* tcgen05 kind::f16 with fp16 operands (power-of-two scaled
@@ -221,7 +229,8 @@ igafd_status igafd_apply_A(igafd_patch *patch, const double *x_dev,
 /* z = P^{-1} r by fast diagonalization (Algorithm 1 in 2D, Algorithm 3 in
  * 3D, with the forward step applying U_k^T and the backward step U_k):
  * forward mode-k products, divide by D_1 (+) ... (+) D_d, backward mode-k
- * products. With IGAFD_FP64 the result equals P^{-1} r up to rounding;
+ * products. With IGAFD_FP64 the result equals P^{-1} r up to rounding (an
+ * entry that is not finite makes the whole contracted row NaN);
  * other dtypes give an inexact P^{-1}. The tensor-core dtypes (BF16, FP16,
  * TF32) need n_k <= 256 and return IGAFD_ERR_ARG otherwise. IGAFD_ADI
  * applies P_J^{-1} as igafd_apply_prec_adi does. r_dev and z_dev must not

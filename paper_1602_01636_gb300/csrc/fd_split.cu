@@ -1,4 +1,6 @@
-// FP64 fast-diagonalization apply on the tensor cores, for n_k <= 256.
+// FP64 fast-diagonalization apply on the tensor cores, for n_k <= 256 (in
+// directions whose U_k has rows of very different sizes on the FP64 pipe, see
+// kRowRange).
 //
 // GB300 issues two FP64 FMAs per clock per SM (1.26 TFLOP/s in all), so the
 // 12 n^4 FLOP of the six mode products take 2.6 ms at n = 128 on the FP64
@@ -24,7 +26,7 @@
 // multiplies the integer result before that rounding. No FP64 instruction is
 // executed (each would issue at the 2-per-clock rate).
 //
-// Measured: 207 us per apply at n = 128 (SIMT: 3.10 ms), 108 us at (95, 61, 77)
+// Measured: 207 us per apply at n = 128 (SIMT: 3.10 ms), 110 us at (95, 61, 77)
 // (SIMT: 0.98 ms). A pass at n = 128 takes the phases of its one tile per SM in
 // turn: reading and splitting the rows (6 us), the MMAs with the summation of
 // their accumulators (the MMAs alone 5 us), the last rounding (2.5 us), and
@@ -78,6 +80,9 @@ struct SplitArgs {
   int N, Np, NT;          // columns, padded to 16; columns per CTA (multiple of 16)
   const unsigned char *img;   // digits of B: [slice][64-wide K chunk][Np][128 B], swizzled
   const int *eb;              // exponent field of each row of B
+  const int *range;           // largest and smallest exponent field of the rows of U_k
+  const double *U;            // U_k, B's element (column j, term k) at j u_j + k u_k
+  int u_j, u_k;
   const double *inv_lam;      // divide table, indexed like out (null: none)
   const double *done;
   int *err;
@@ -134,14 +139,15 @@ __device__ __forceinline__ int exp_field(uint32_t hi) {
 }
 
 // X + kBias with X = d 2^(1022 + kBits - ea) rounded down, |X| <= 2^kBits, as
-// its upper and lower 30 bits (junk above bit 30 of the lower word).
-__device__ __forceinline__ void biased_fixed(double d, int ea, uint32_t &w1, uint32_t &w0) {
+// its upper and lower 30 bits (junk above bit 30 of the lower word); d's
+// exponent field lowered by s (0 or a column scaling of U_k).
+__device__ __forceinline__ void biased_fixed(double d, int ea, uint32_t &w1, uint32_t &w0, int s = 0) {
   const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
   // mantissa with the hidden bit at bit 63 (its place holds the exponent's
   // lowest bit, which is 0 where there is no hidden bit)
   const uint32_t mh = __funnelshift_l(lo, hi, 11) | ((hi & 0x7ff00000u) ? 0x80000000u : 0u);
   const uint32_t ml = lo << 11;
-  const uint32_t sh = (uint32_t)(ea + 64 - kBits - exp_field(hi));
+  const uint32_t sh = (uint32_t)(ea + 64 - kBits - exp_field(hi) + s);
   const uint32_t s1 = min(sh, 32u);
   uint32_t xh = shr_clamp(mh, s1);
   uint32_t xl = shr_clamp(__funnelshift_rc(ml, mh, s1), sh - s1);
@@ -226,13 +232,61 @@ template <int N, typename F> __device__ __forceinline__ void each_step(F &&f) {
   each_of(f, std::make_integer_sequence<int, N>{});
 }
 
+// Largest difference between the exponents of the rows of U_k (by their largest
+// entries) up to which the digits are used: a right-hand side that meets a
+// small row multiplies entries that lost as many bits of the 58 as the row is
+// smaller than the columns' largest. Uniform knots have at most 3 (n <= 256,
+// every degree), spans graded by up to 50 have 4, span scalings 4 for a
+// standard deviation of 1 of their logarithms. Largest errors of P^{-1} r in 2D
+// over random, constant and single-entry right-hand sides (60 graded and scaled
+// pencils), digits against FP64 chains: 0.9 and 2.5 x 1e-15 up to 4, 2.5 and
+// 2.0 at 5, 19 and 1.5 at 8.
+constexpr int kRowRange = 4;
+
+// The mode product of this CTA's rows and columns as FP64 chains, for
+// pencils beyond that range and for U_k that is not finite: on the FP64 pipe,
+// rows and columns as below, U_k from L1 (n = 128: 3.1 ms per apply, as the
+// SIMT kernel; (95, 61, 77): 0.70 ms). Decided by what the set-up left on the
+// device, so that captured launches follow a new set-up.
+template <bool LAM>
+__device__ __forceinline__ void chain_rows(const SplitArgs &a, int n0, int cols) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long m = (long long)blockIdx.x * kM + (warp & 3) * 32 + lane;
+  if (m >= a.M) return;
+  const long long hi = m / a.F, lo = m - hi * a.F;
+  const double *src = a.in + hi * a.in_hi + lo * a.in_lo;
+  const long long ob = hi * a.out_hi + lo * a.out_lo;
+  constexpr int C = 8;                                     // columns at a time
+  for (int c = C * (warp >> 2); c < cols; c += C * (kWarps / 4)) {
+    double acc[C];
+    const double *u[C];
+#pragma unroll
+    for (int t = 0; t < C; ++t) {
+      acc[t] = 0.0;
+      u[t] = a.U + (size_t)min(n0 + c + t, a.N - 1) * a.u_j;
+    }
+    for (int k = 0; k < a.K; ++k) {
+      const double x = __ldg(src + (long long)k * a.in_k);
+#pragma unroll
+      for (int t = 0; t < C; ++t) acc[t] = fma(x, __ldg(u[t] + (size_t)k * a.u_k), acc[t]);
+    }
+#pragma unroll
+    for (int t = 0; t < C; ++t)
+      if (c + t < cols && n0 + c + t < a.N) {
+        const long long o = ob + (long long)(n0 + c + t) * a.out_n;
+        a.out[o] = LAM ? acc[t] * __ldg(a.inv_lam + o) : acc[t];
+      }
+  }
+}
+
 template <int KP, bool LAM>
 __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(SplitArgs a) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char *sB = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ uint64_t bar_b[2], bar_full[2], bar_empty[2];
   __shared__ uint32_t tmem_slot;
-  __shared__ unsigned short s_ea[4][kM], s_eb[kM];
+  __shared__ unsigned short s_ea[4][kM];
+  __shared__ short s_eb[kM];
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = (int)blockIdx.y * a.NT;
@@ -291,8 +345,9 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     if (lane == 0) load_slices(0, kFirst, &bar_b[0]);
   }
+  const int rows_hi = a.range[0], rows_lo = a.range[1];
   for (int n = tid; n < NTc; n += kThreads)
-    s_eb[n] = (unsigned short)(n0 + n < a.N ? a.eb[n0 + n] : 1);
+    s_eb[n] = (short)(n0 + n < a.N ? a.eb[n0 + n] : 1);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -301,6 +356,15 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
   pdl_wait();
   pdl_trigger();
   if (a.done && *a.done != 0.0) {                          // uniform
+    if (tid == 0) wait_on(&bar_b[0], 0, &s_fail);
+    __syncthreads();
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmem));
+    return;
+  }
+
+  if (rows_hi - rows_lo > kRowRange || rows_hi == 0x7ff) {  // uniform
+    chain_rows<LAM>(a, n0, NTc);
     if (tid == 0) wait_on(&bar_b[0], 0, &s_fail);
     __syncthreads();
     if (warp == 0)
@@ -578,36 +642,72 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
 
 // Digits of B = U_k^T (transpose) or U_k as the shared-memory images of the
 // pass kernel, and the exponent field of each row: one CTA per (row, image).
+// U_k's columns are brought to one size by powers of two s_j first (outlier
+// eigenvectors are large at the ends, 2^4.4 times the others at n = 128, p = 3,
+// and would take those bits from the rest of a row): the forward product's
+// column j is raised by s_j, U_k's lowered; between the two only the range of
+// the intermediate values moves, by 2^4 or so. Without it constant right-hand
+// sides at n = 120, p = 7 were off by 1.2e-14 (FP64 chains 1.8e-15, now 0.4e-15).
+// The forward images are made first.
 struct ImgJob {
   const double *U;
   int n, Np, Kp, transpose;
   unsigned char *img;
   int *eb;
+  int *col;       // s_j, set by the forward image
+  int *range;     // largest and smallest exponent field of U_k's rows
 };
 struct ImgBatch {
-  ImgJob j[6];
+  ImgJob j[3];
 };
 __global__ void __launch_bounds__(256) split_image_kernel(ImgBatch b) {
   const ImgJob J = b.j[blockIdx.y];
   const int r = blockIdx.x, k = threadIdx.x;
   if (r >= J.Np) return;
-  __shared__ int s_e[8];
+  __shared__ int s_e[2][8];
   const int nkc = (J.Kp + 63) >> 6;
   double d = 0.0;
-  if (r < J.n && k < J.n) d = J.transpose ? J.U[(size_t)k * J.n + r] : J.U[(size_t)r * J.n + k];
-  int e = exp_field((uint32_t)__double2hiint(d));
-  for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-  if ((k & 31) == 0) s_e[k >> 5] = e;
+  int s = 0;
+  if (r < J.n && k < J.n) {
+    d = J.transpose ? J.U[(size_t)k * J.n + r] : J.U[(size_t)r * J.n + k];
+    if (!J.transpose) s = J.col[k];
+  }
+  int raw = exp_field((uint32_t)__double2hiint(d)), e = raw - s;
+  for (int o = 16; o > 0; o >>= 1) {
+    raw = max(raw, __shfl_xor_sync(0xffffffffu, raw, o));
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+  }
+  if ((k & 31) == 0) {
+    s_e[0][k >> 5] = raw;
+    s_e[1][k >> 5] = e;
+  }
   __syncthreads();
-  for (int w = 0; w < 8; ++w) e = max(e, s_e[w]);
-  if (k == 0) J.eb[r] = e;
+  for (int w = 0; w < 8; ++w) {
+    raw = max(raw, s_e[0][w]);
+    e = max(e, s_e[1][w]);
+  }
+  if (k == 0 && J.transpose) {
+    const int up = r < J.n ? max(-64, min(64, e - 1023)) : 0;
+    if (r < J.n) J.col[r] = up;
+    J.eb[r] = e + up;
+    if (r == 0) {
+      J.range[0] = 0;
+      J.range[1] = 0x7ff;
+    }
+  } else if (k == 0) {
+    J.eb[r] = e;
+    if (r < J.n) {
+      atomicMax(&J.range[0], raw);
+      atomicMin(&J.range[1], raw);
+    }
+  }
   if (k >= nkc * 64) return;
   uint32_t w1, w0;
-  biased_fixed(d, e, w1, w0);
+  biased_fixed(d, e, w1, w0, s);
   const int kb = (k & 63) * 2;
   unsigned char *at = J.img + ((size_t)(k >> 6) * J.Np + r) * 128 + ((((kb >> 4) ^ (r & 7)) << 4) | (kb & 15));
   const size_t slice = (size_t)nkc * J.Np * 128;
-  auto put = [&](int s, uint32_t w) { *reinterpret_cast<unsigned short *>(at + s * slice) = (unsigned short)w; };
+  auto put = [&](int i, uint32_t w) { *reinterpret_cast<unsigned short *>(at + i * slice) = (unsigned short)w; };
   put(0, digit2<2>(w1, w1));
   put(1, digit2<1>(w1, w1));
   put(2, digit2<0>(w1, w1));
@@ -629,6 +729,7 @@ size_t pass_smem(int Kp) {
 struct FDSplit {
   unsigned char *img[3][2];   // [direction][0: U_k^T, 1: U_k]
   int *eb[3][2];
+  int *col[3];                // column scalings of U_k (exponents), then its rows' range (2)
 };
 
 bool igafd_fd_split_shape(const igafd_patch *P) {
@@ -638,19 +739,24 @@ bool igafd_fd_split_shape(const igafd_patch *P) {
 }
 
 // Digit images of U_k^T and U_k. Allocates on the first call; later calls (a
-// re-setup of P) refill the same buffers. Enqueues one kernel.
+// re-setup of P) refill the same buffers. Enqueues two kernels.
 igafd_status igafd_fd_split_init(igafd_patch *P, cudaStream_t s) {
   if (!igafd_fd_split_shape(P)) return IGAFD_OK;
   if (!P->split) {
     P->split = (FDSplit *)calloc(1, sizeof(FDSplit));
     if (!P->split) return IGAFD_ERR_OOM;
   }
-  ImgBatch b{};
-  int jobs = 0, rows = 0;
-  for (int k = 0; k < P->dim; ++k)
+  ImgBatch b[2] = {};
+  int rows = 0;
+  for (int k = 0; k < P->dim; ++k) {
+    const int n = P->n[k];
+    if (!P->split->col[k] && cudaMalloc(&P->split->col[k], (n + 2) * sizeof(int)) != cudaSuccess) {
+      cudaGetLastError();
+      return IGAFD_ERR_OOM;
+    }
     for (int d = 0; d < 2; ++d) {
-      ImgJob &J = b.j[jobs++];
-      J.U = P->U[k]; J.n = P->n[k]; J.Np = pad(P->n[k], 16); J.Kp = pad(P->n[k], 32);
+      ImgJob &J = b[d].j[k];
+      J.U = P->U[k]; J.n = n; J.Np = pad(n, 16); J.Kp = pad(n, 32);
       J.transpose = d == 0;
       const size_t sz = (size_t)kSlices * ((J.Kp + 63) / 64) * J.Np * 128;
       if ((!P->split->img[k][d] && cudaMalloc(&P->split->img[k][d], sz) != cudaSuccess) ||
@@ -660,21 +766,26 @@ igafd_status igafd_fd_split_init(igafd_patch *P, cudaStream_t s) {
       }
       J.img = P->split->img[k][d];
       J.eb = P->split->eb[k][d];
+      J.col = P->split->col[k];
+      J.range = J.col + n;
       rows = J.Np > rows ? J.Np : rows;
     }
-  split_image_kernel<<<dim3(rows, jobs), 256, 0, s>>>(b);
-  IGAFD_LAUNCHED(1);
+  }
+  for (int d = 0; d < 2; ++d) split_image_kernel<<<dim3(rows, P->dim), 256, 0, s>>>(b[d]);
+  IGAFD_LAUNCHED(2);
   IGAFD_CUDA(cudaGetLastError());
   return IGAFD_OK;
 }
 
 void igafd_fd_split_free(igafd_patch *P) {
   if (!P || !P->split) return;
-  for (int k = 0; k < 3; ++k)
+  for (int k = 0; k < 3; ++k) {
     for (int d = 0; d < 2; ++d) {
       cudaFree(P->split->img[k][d]);
       cudaFree(P->split->eb[k][d]);
     }
+    cudaFree(P->split->col[k]);
+  }
   free(P->split);
   P->split = nullptr;
 }
@@ -686,6 +797,10 @@ static igafd_status launch_pass(igafd_patch *P, int k, int dir, SplitArgs a, cud
   a.Np = pad(a.N, 16);
   a.img = P->split->img[k][dir];
   a.eb = P->split->eb[k][dir];
+  a.range = P->split->col[k] + P->n[k];
+  a.U = P->U[k];
+  a.u_j = dir == 0 ? 1 : a.N;
+  a.u_k = dir == 0 ? a.N : 1;
   a.err = P->err_flag;
   // Column split: with fewer 128-row tiles than SMs, a CTA's columns are
   // halved while all CTAs still fit one wave (a CTA's time is about half the
