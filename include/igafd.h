@@ -234,7 +234,8 @@ igafd_status igafd_apply_A(igafd_patch *patch, const double *x_dev,
  * other dtypes give an inexact P^{-1}. The tensor-core dtypes (BF16, FP16,
  * TF32) need n_k <= 256 and return IGAFD_ERR_ARG otherwise. IGAFD_ADI
  * applies P_J^{-1} as igafd_apply_prec_adi does. r_dev and z_dev must not
- * overlap. */
+ * overlap. A device wait that runs out is not reported here; the FP64 FD
+ * leaves NaN in z then (igafd_set_wait_polls). */
 igafd_status igafd_apply_prec(igafd_patch *patch, igafd_dtype dtype,
                               const double *r_dev, double *z_dev, void *stream);
 
@@ -415,6 +416,13 @@ igafd_status igafd_setup_prec(igafd_patch *patch, void *stream);
  * of its diagonal; FP64 cyclic Jacobi otherwise; 1 = FP64 Jacobi for every direction. igafd_patch_info.eig_refined reports the
  * route each direction took. Other values: IGAFD_ERR_ARG. */
 igafd_status igafd_set_eig_route(igafd_patch *patch, int route);
+
+/* Polls after which a device wait of the FP64 FD on the tensor cores gives up
+ * (default 2^26, some seconds; negative or larger: the default; 0: every wait
+ * gives up at once). Such a wait leaves NaN in the entries of z that it stands
+ * for; solves also report an error. Launches captured before the call keep
+ * their limit. */
+igafd_status igafd_set_wait_polls(igafd_patch *patch, long long polls);
 
 /* Condition estimate of P^{-1} A from the last PCG solve on this patch (the
  * CG-Lanczos relation: with the recorded step lengths alpha_j and direction

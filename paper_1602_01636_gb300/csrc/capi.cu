@@ -174,6 +174,12 @@ extern "C" igafd_status igafd_setup_prec(igafd_patch *P, void *stream) {
   return igafd_build_prec(P, (cudaStream_t)stream);
 }
 
+extern "C" igafd_status igafd_set_wait_polls(igafd_patch *P, long long polls) {
+  if (!P) return IGAFD_ERR_ARG;
+  P->wait_polls = polls < 0 || polls > kWaitPolls ? kWaitPolls : (int)polls;
+  return IGAFD_OK;
+}
+
 extern "C" igafd_status igafd_set_eig_route(igafd_patch *P, int route) {
   if (!P || (route != 0 && route != 1)) return IGAFD_ERR_ARG;
   P->eig_route = route;
@@ -219,6 +225,7 @@ extern "C" igafd_status igafd_setup_patch(const igafd_patch_desc *d, void *strea
   P->kappa_p = d->kappa_ctrl ? d->kappa_p : 0;
   P->kappa = d->kappa;
   P->fd_fused = 1;
+  P->wait_polls = kWaitPolls;
   for (int o = 0; o < 3; ++o) P->fd_fused_op[o] = 1;
   if (cudaGetDevice(&P->dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, P->dev) != cudaSuccess) {

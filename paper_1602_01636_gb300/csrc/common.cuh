@@ -71,6 +71,8 @@ enum {
   S_COUNT
 };
 
+constexpr int kWaitPolls = 1 << 26;   // polls of a bounded device wait (some seconds)
+
 struct FDMixed;   // mixed-precision FD workspace (fd_tc.cu)
 struct FDSplit;   // digit images of the FP64 FD on the tensor cores (fd_split.cu)
 
@@ -120,7 +122,7 @@ struct igafd_patch {
   long long loop_nodes;         // kernels per replay
   unsigned long long *tstat;    // stencil timing on the device: [0] earliest block start
                                 // of the running launch, [1] summed ns, [2] launches
-  int loop_key[13];             // dtype, flexible, true_every, chunk, valid, FD form (2),
+  int loop_key[14];             // dtype, flexible, true_every, chunk, valid, FD form (2),
                                 // stencil depth, stencil rows, FD tile shape (4)
   double *partial;              // [PARTIAL_SLOTS][MAX_BLOCKS]
   unsigned int *counter;        // last-block counters
@@ -148,6 +150,7 @@ struct igafd_patch {
   // diagnostics
   double min_detJ, q_bound, setup_ms, eig_ms;
   int *err_flag;                // device error flags from setup kernels
+  int wait_polls;               // of the FP64 FD's waits (igafd_set_wait_polls)
   void *adi;                    // three-variable ADI preconditioner state (adi.cu), or null
 };
 

@@ -26,7 +26,7 @@
 // multiplies the integer result before that rounding. No FP64 instruction is
 // executed (each would issue at the 2-per-clock rate).
 //
-// Measured: 207 us per apply at n = 128 (SIMT: 3.10 ms), 110 us at (95, 61, 77)
+// Measured: 212 us per apply at n = 128 (SIMT: 3.10 ms), 110 us at (95, 61, 77)
 // (SIMT: 0.98 ms). A pass at n = 128 takes the phases of its one tile per SM in
 // turn: reading and splitting the rows (6 us), the MMAs with the summation of
 // their accumulators (the MMAs alone 5 us), the last rounding (2.5 us), and
@@ -64,7 +64,7 @@ using namespace igafd_split;
 constexpr int kM = 128;                 // rows per CTA (MMA M, TMEM lanes)
 constexpr int kThreads = 512;           // 4 warps per lane quarter
 constexpr int kWarps = kThreads / 32;
-constexpr long long kSpin = 1ll << 26;  // bounded waits
+constexpr int kSpin = kWaitPolls;    // bounded waits
 // X + kBias = sum_s (digit_s + 512) 1024^(5-s): every 10-bit field is then the
 // digit plus 512
 constexpr unsigned long long kBias = 512ull * (1ull + (1ull << 10) + (1ull << 20) + (1ull << 30) +
@@ -86,6 +86,7 @@ struct SplitArgs {
   const double *inv_lam;      // divide table, indexed like out (null: none)
   const double *done;
   int *err;
+  int polls;              // of a wait before it gives up
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -104,8 +105,9 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
 }
 
 // Bounded wait, given up early once another thread's wait ran out.
-__device__ __forceinline__ bool wait_on(uint64_t *bar, uint32_t parity, const int *failed) {
-  for (long long it = 0; it < kSpin; ++it) {
+__device__ __forceinline__ bool wait_on(uint64_t *bar, uint32_t parity, const int *failed,
+                                        int polls = kSpin) {
+  for (int it = 0; it < polls; ++it) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
   __shared__ uint32_t tmem_slot;
   __shared__ unsigned short s_ea[4][kM];
   __shared__ short s_eb[kM];
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_issued[2];     // commits on bar_full
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = (int)blockIdx.y * a.NT;
   const int NTc = a.Np - n0 < a.NT ? a.Np - n0 : a.NT;     // columns of this CTA
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
       mbar_init(&bar_empty[i], kWarps);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_fail = 0;
+    s_fail = s_issued[0] = s_issued[1] = 0;
   }
   auto load_slices = [&](int s0, int s1, uint64_t *bar) {   // one thread
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
@@ -494,10 +496,10 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     const int buf = st & 1;
     if (sub == 0) {                                        // (a poll each once they have arrived)
       constexpr unsigned waits = step_waits(KP, p.g);
-      if (waits & 1u) ok = ok && wait_on(&bar_b[0], 0, &s_fail);
-      if (waits & 2u) ok = ok && wait_on(&bar_b[1], 0, &s_fail);
+      if (waits & 1u) ok = ok && wait_on(&bar_b[0], 0, &s_fail, a.polls);
+      if (waits & 2u) ok = ok && wait_on(&bar_b[1], 0, &s_fail, a.polls);
     }
-    if (st >= 2) ok = ok && wait_on(&bar_empty[buf], (uint32_t)(((st >> 1) - 1) & 1), &s_fail);
+    if (st >= 2) ok = ok && wait_on(&bar_empty[buf], (uint32_t)(((st >> 1) - 1) & 1), &s_fail, a.polls);
     ok = __all_sync(0xffffffffu, ok);
     if (!ok) return;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -527,6 +529,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
           "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
               smem_u32(&bar_full[buf]))
           : "memory");
+      s_issued[buf] = (st >> 1) + 1;
     }
     __syncwarp();
   };
@@ -538,7 +541,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
   int st = 0;
   if (warp == 0) issue(std::integral_constant<int, 0>{}, std::integral_constant<int, 0>{}, 0, 0);
   for (int sub = 0; sub < nsub; ++sub) {
-    long long T[C];
+    long long T[C] = {};
     auto sum = [&](auto part, auto step) {
       constexpr int i = decltype(step)::value, part_ = decltype(part)::value;
       constexpr int KT = part_ ? KR : KA, per = Steps<KT>::kCount;
@@ -546,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
       const int buf = st & 1;
       if (warp == ((st + 1) & (kWarps - 1)) && (i + 1 < per || (KR == 0 && sub + 1 < nsub)))
         issue(part, std::integral_constant<int, (i + 1) % per>{}, i + 1 < per ? sub : sub + 1, st + 1);
-      ok = ok && wait_on(&bar_full[buf], (uint32_t)((st >> 1) & 1), &s_fail);
+      ok = ok && wait_on(&bar_full[buf], (uint32_t)((st >> 1) & 1), &s_fail, a.polls);
       ok = __all_sync(0xffffffffu, ok);
       ++st;
       if (!ok) {
@@ -599,14 +602,15 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
       if (warp == (st & (kWarps - 1))) issue(second, std::integral_constant<int, 0>{}, 0, st);
       sum_part(second);
     }
-    if (!ok || !row_ok) continue;
+    if (!row_ok) continue;
     const int nl0 = sub * kNS + kq * C;                  // this thread's first column, and how many
     const int ncol = min(C, min(NTc - nl0, a.N - n0 - nl0));
     const long long o0 = ob + (long long)(n0 + nl0) * a.out_n;
     double lam[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) lam[c] = LAM && c < ncol ? __ldg(a.inv_lam + o0 + c * a.out_n) : 1.0;
-    bool slow = bad_row;
+    const bool bad = bad_row || !ok;                     // !ok: NaN, never what the buffer held before
+    bool slow = bad;
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       const double y = round_fixed<LAM>(T[c], ea + (int)s_eb[(nl0 + c) & (kM - 1)] - 2060 - kTop, lam[c], slow);
@@ -617,7 +621,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
       for (int c = 0; c < C; ++c)
         if (c < ncol)
           a.out[o0 + c * a.out_n] =
-              bad_row ? __longlong_as_double(0x7ff8000000000000ll)
+              bad ? __longlong_as_double(0x7ff8000000000000ll)
                       : round_slow(T[c], ea + (int)s_eb[nl0 + c] - 2060 - kTop, lam[c]);
     }
   }
@@ -630,11 +634,9 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(KP)) split_pass_kernel(S
     // finish before shared memory and TMEM are released
     const int none = 0;
     wait_on(&bar_b[0], 0, &none);
-    wait_on(&bar_b[1], 0, &none);
-    for (int i = 0; i < 2; ++i) {
-      wait_on(&bar_full[i], 0, &none);
-      wait_on(&bar_full[i], 1, &none);
-    }
+    if (kFirst < kSlices) wait_on(&bar_b[1], 0, &none);
+    for (int i = 0; i < 2; ++i)
+      if (s_issued[i]) wait_on(&bar_full[i], (uint32_t)((s_issued[i] - 1) & 1), &none);
   }
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmem));
@@ -802,6 +804,7 @@ static igafd_status launch_pass(igafd_patch *P, int k, int dir, SplitArgs a, cud
   a.u_j = dir == 0 ? 1 : a.N;
   a.u_k = dir == 0 ? a.N : 1;
   a.err = P->err_flag;
+  a.polls = P->wait_polls;
   // Column split: with fewer 128-row tiles than SMs, a CTA's columns are
   // halved while all CTAs still fit one wave (a CTA's time is about half the
   // splitting of its rows, which every column part repeats, and half the

@@ -506,7 +506,7 @@ static igafd_status loop_graph(igafd_patch *P, igafd_dtype dt, int flex, int tru
   // everything that selects the captured kernels: the FD form and the stencil
   // pipeline too (set by the autotuner or explicitly between solves)
   const int op = dt == IGAFD_TF32 ? 0 : dt == IGAFD_BF16 ? 1 : 2;
-  const int key[13] = {(int)dt, flex, true_every, chunk, 1 + timing, P->fd_fused,
+  const int key[14] = {(int)dt, flex, true_every, chunk, 1 + timing, P->wait_polls, P->fd_fused,
                        P->fd_fused_op[op], P->stencil_stages, P->stencil_rows, P->fd_tile[op][0],
                        P->fd_tile[op][1], P->fd_tile[op][2], P->fd_tile[op][3]};
   if (P->loop_exec && memcmp(key, P->loop_key, sizeof(key)) == 0) return IGAFD_OK;

@@ -76,6 +76,7 @@ EXPORTS = ["igafd_setup_patch", "igafd_destroy_patch", "igafd_patch_query", "iga
            "igafd_pcg_solve", "igafd_pcg_default_opts", "igafd_status_str",
            "igafd_kernel_launches", "igafd_batch_pcg_solve", "igafd_autotune",
            "igafd_set_stencil_stages", "igafd_set_stencil_rows", "igafd_setup_prec", "igafd_set_eig_route",
+           "igafd_set_wait_polls",
            "igafd_pcg_condition_estimate", "igafd_lanczos_extremes", "igafd_set_fd_fused", "igafd_scaling_rows", "igafd_patch_features",
            "igafd_patch_sepfit", "igafd_set_scalings", "igafd_mlp_create", "igafd_mlp_destroy",
            "igafd_mlp_set_normalization", "igafd_mlp_get_params", "igafd_mlp_set_params",
@@ -134,6 +135,7 @@ def lib():
     L.igafd_pcg_condition_estimate.argtypes = [vp, C.c_int, dp, dp, dp]
     L.igafd_lanczos_extremes.argtypes = [dp, dp, C.c_int, dp, dp]
     L.igafd_set_eig_route.argtypes = [vp, C.c_int]
+    L.igafd_set_wait_polls.argtypes = [vp, C.c_longlong]
     L.igafd_scaling_rows.argtypes = [vp, C.POINTER(C.c_int)]
     L.igafd_patch_features.argtypes = [vp, vp, vp]
     L.igafd_patch_sepfit.argtypes = [vp, C.c_int, vp, vp]
@@ -539,6 +541,11 @@ class Patch:
         """0: FP32 start + FP64 refinement (default); 1: FP64 Jacobi.
         Takes effect at the next setup_prec()."""
         _check(lib().igafd_set_eig_route(self.h, int(route)), "set_eig_route")
+
+    def set_wait_polls(self, polls=-1):
+        """Polls after which a device wait of the FP64 FD gives up and leaves NaN
+        (0: at once, negative: the default)."""
+        _check(lib().igafd_set_wait_polls(self.h, int(polls)), "set_wait_polls")
 
     def set_stencil_rows(self, rows):
         _check(lib().igafd_set_stencil_rows(self.h, int(rows)), "set_stencil_rows")

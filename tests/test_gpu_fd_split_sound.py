@@ -114,3 +114,25 @@ def test_eigenvector_images_follow_the_scalings():
     patch.set_scalings(None)
     assert torch.equal(patch.apply_prec(b), z0) and torch.equal(patch.pcg(b, tol=1e-10)[0], x0)
     patch.close()
+
+
+# one and two parts, one and two column blocks, the early slices of each length
+@pytest.mark.parametrize("dim,n,p", [(3, (20, 33, 8), 2), (2, (96, 128), 3), (2, (200, 129), 2)])
+def test_waits_that_give_up(dim, n, p):
+    """Every wait gives up at once: NaN in place of what the buffers held, an
+    error from a solve, and a patch that works as before afterwards."""
+    torch = need_gpu()
+    from paper_1602_01636_gb300 import igafd
+    patch = igafd.Patch.from_problem(synth.Problem(dim, n, p))
+    r = to_dev(np.random.default_rng(6).standard_normal(patch.N))
+    want = patch.apply_prec(r).clone()
+    patch.set_wait_polls(0)
+    assert torch.isnan(patch.apply_prec(r)).all().item()
+    with pytest.raises(igafd.IgafdError):
+        patch.pcg(r)
+    patch.set_wait_polls()
+    assert torch.equal(patch.apply_prec(r), want)
+    fresh = igafd.Patch.from_problem(synth.Problem(dim, n, p))
+    assert torch.equal(patch.pcg(r)[0], fresh.pcg(r)[0])
+    patch.close()
+    fresh.close()
