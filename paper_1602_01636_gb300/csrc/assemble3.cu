@@ -35,6 +35,7 @@
 #include "geom.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -46,6 +47,20 @@ using namespace igafd_geom;
 constexpr int kThr = 128;
 constexpr int kLoad = 64;       // points of direction 1 per block of load_kernel
 constexpr int kRows = 64;       // rows per block of dir1_kernel (small patches fill more of it)
+constexpr int kMaxSmem = 200 * 1024;   // dynamic shared memory that a kernel may ask for
+
+// Lets a kernel ask for up to kMaxSmem, once per device: the attribute belongs
+// to the kernel, not to a launch, and other host threads launch it too.
+template <typename Kern> igafd_status allow_smem(Kern kern, std::atomic<unsigned long long> &set) {
+  int dev = 0;
+  IGAFD_CUDA(cudaGetDevice(&dev));
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (!(set.load() & bit)) {
+    IGAFD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    set.fetch_or(bit);
+  }
+  return IGAFD_OK;
+}
 
 // order-preserving map of doubles to unsigned integers
 __host__ __device__ __forceinline__ unsigned long long key_of(double d) {
@@ -514,8 +529,9 @@ igafd_status load_p(const PV &v, const double *fq, double *b, cudaStream_t s) {
   constexpr int A = P + 1, TE = kLoad / A;
   const size_t smem = sizeof(double) * std::max((size_t)9 * v.gm[0] * RG, (size_t)A * A * kLoad);
   if constexpr (RG > 1)
-    if (smem > 200 * 1024) return load_p<P, 1>(v, fq, b, s);
-  IGAFD_CUDA(cudaFuncSetAttribute((load_kernel<P, RG>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > kMaxSmem) return load_p<P, 1>(v, fq, b, s);
+  static std::atomic<unsigned long long> smem_set{0};
+  IGAFD_TRY(allow_smem(load_kernel<P, RG>, smem_set));
   const int tiles = (v.nel[0] + TE - 1) / TE;
   for (int c3 = 0; c3 < std::min(A, v.nel[2]); ++c3)
     for (int c2 = 0; c2 < std::min(A, v.nel[1]); ++c2)
@@ -620,7 +636,8 @@ struct Runner {
     a.H = P->stencil_half ? P->sh_H : 0;
     const int km = P->kctrl ? P->dir[0].km : 0;
     const size_t smem0 = (size_t)(9 * P->dir[0].gm + km) * sizeof(double);
-    IGAFD_CUDA(cudaFuncSetAttribute(points_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0));
+    static std::atomic<unsigned long long> smem_set{0};
+    IGAFD_TRY(allow_smem(points_kernel, smem_set));
     size_t smem1 = 0;                       // rows' points of a dir1 block
     for (int i = 0; i < P->n[0]; i += kRows) {
       int lo, hi;
