@@ -103,6 +103,10 @@ struct AsmArgs {
 // One row (q2, q3) of points per block: the geometry's control net contracted
 // in directions 2 and 3 into rows over direction 1's control points (values,
 // and derivatives in directions 2 and 3), then per point along direction 1.
+// ROWS false: nets whose rows do not fit in shared memory (more than about 2800
+// control points of direction 1, far more than the points), each point's map
+// straight from the net.
+template <bool ROWS>
 __global__ void __launch_bounds__(kThr) points_kernel(AsmArgs a, int e3lo) {
   extern __shared__ double sm[];
   const PV &v = a.v;
@@ -110,7 +114,7 @@ __global__ void __launch_bounds__(kThr) points_kernel(AsmArgs a, int e3lo) {
   const int ql = blockIdx.x, q2 = a.q2lo + ql, q3 = e3lo * nq + blockIdx.y;
   double *row = sm;                         // [3 coordinates][vv, dv, vd][gm]
   double *krow = sm + 9 * gm;               // [km]
-  {
+  if constexpr (ROWS) {
     const double *v2 = v.gv[1] + (size_t)q2 * ga, *d2 = v.gd[1] + (size_t)q2 * ga;
     const double *v3 = v.gv[2] + (size_t)q3 * ga, *d3 = v.gd[2] + (size_t)q3 * ga;
     const int g2 = v.gspan[1][q2] - gp, g3 = v.gspan[2][q3] - gp;
@@ -161,24 +165,30 @@ __global__ void __launch_bounds__(kThr) points_kernel(AsmArgs a, int e3lo) {
   double *out = a.Q + (size_t)slot * plane + (size_t)ql * a.T1;
   const size_t comp = (size_t)a.ring * nq * plane;
   for (int q1 = threadIdx.x; q1 < a.T1; q1 += kThr) {
-    const double *v1 = v.gv[0] + (size_t)q1 * ga, *d1 = v.gd[0] + (size_t)q1 * ga;
-    const int g1 = v.gspan[0][q1] - gp;
-    double J[3][3] = {};
-    for (int i = 0; i < ga; ++i) {
-      const double x = v1[i], d = d1[i];
+    double J[3][3] = {}, kap = v.kappa;
+    if constexpr (ROWS) {
+      const double *v1 = v.gv[0] + (size_t)q1 * ga, *d1 = v.gd[0] + (size_t)q1 * ga;
+      const int g1 = v.gspan[0][q1] - gp;
+      for (int i = 0; i < ga; ++i) {
+        const double x = v1[i], d = d1[i];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        J[c][0] = fma(row[(c * 3 + 0) * gm + g1 + i], d, J[c][0]);
-        J[c][1] = fma(row[(c * 3 + 1) * gm + g1 + i], x, J[c][1]);
-        J[c][2] = fma(row[(c * 3 + 2) * gm + g1 + i], x, J[c][2]);
+        for (int c = 0; c < 3; ++c) {
+          J[c][0] = fma(row[(c * 3 + 0) * gm + g1 + i], d, J[c][0]);
+          J[c][1] = fma(row[(c * 3 + 1) * gm + g1 + i], x, J[c][1]);
+          J[c][2] = fma(row[(c * 3 + 2) * gm + g1 + i], x, J[c][2]);
+        }
       }
-    }
-    double kap = v.kappa;
-    if (v.kctrl) {
-      const int ka = v.kp + 1, k1 = v.kspan[0][q1] - v.kp;
-      double s = 0.0;
-      for (int i = 0; i < ka; ++i) s = fma(krow[k1 + i], v.kv[0][(size_t)q1 * ka + i], s);
-      kap *= s;
+      if (v.kctrl) {
+        const int ka = v.kp + 1, k1 = v.kspan[0][q1] - v.kp;
+        double s = 0.0;
+        for (int i = 0; i < ka; ++i) s = fma(krow[k1 + i], v.kv[0][(size_t)q1 * ka + i], s);
+        kap *= s;
+      }
+    } else {
+      const int t[3] = {q1, q2, q3};
+      double x[3];
+      geo_eval<3>(v, t, x, J);
+      kap = kappa_eval<3>(v, t);
     }
     // Q = kappa |det| J^-1 J^-T = kappa / |det| (adj J)(adj J)^T; B row r of the adjugate
     double B[3][3];
@@ -415,8 +425,8 @@ __global__ void __launch_bounds__(kRows) dir1_kernel(AsmArgs a) {
 // direction 1 (every other tile); groups of threads share the element's rows
 // (q2, q3), each thread summing its points q1 into the (p + 1)^2 local
 // functions of those directions, with the geometry contracted along rows of points as in points_kernel;
-// direction 1 is contracted last, in shared memory.
-template <int P, int RG>
+// direction 1 is contracted last, in shared memory. (ROWS as in points_kernel.)
+template <int P, int RG, bool ROWS>
 __global__ void __launch_bounds__(kLoad * RG) load_kernel(PV v, int c2, int c3, int ne2, int par,
                                                     const double *fq, double *b) {
   constexpr int A = P + 1, NQ = P + 1, TE = kLoad / NQ;
@@ -442,7 +452,7 @@ __global__ void __launch_bounds__(kLoad * RG) load_kernel(PV v, int c2, int c3, 
     const double *v3 = v.gv[2] + (size_t)q3 * ga, *d3 = v.gd[2] + (size_t)q3 * ga;
     const int g2 = v.gspan[1][q2] - gp, g3 = v.gspan[2][q3] - gp;
     __syncthreads();
-    for (int k = t; k < 3 * G; k += kLoad) {
+    for (int k = t; ROWS && k < 3 * G; k += kLoad) {
       const int c = k / G, g1 = k - c * G;
       double s0 = 0.0, s2 = 0.0, s3 = 0.0;
       for (int a3 = 0; a3 < ga; ++a3) {
@@ -463,19 +473,24 @@ __global__ void __launch_bounds__(kLoad * RG) load_kernel(PV v, int c2, int c3, 
     }
     __syncthreads();
     if (t < np && r + grp < NQ * NQ) {
-      const double *v1 = v.gv[0] + (size_t)q1 * ga, *d1 = v.gd[0] + (size_t)q1 * ga;
-      const int g1 = v.gspan[0][q1] - gp - glo;
       double J[3][3] = {}, X[3] = {};
-      for (int i = 0; i < ga; ++i) {
-        const double x = v1[i], d = d1[i];
+      if constexpr (ROWS) {
+        const double *v1 = v.gv[0] + (size_t)q1 * ga, *d1 = v.gd[0] + (size_t)q1 * ga;
+        const int g1 = v.gspan[0][q1] - gp - glo;
+        for (int i = 0; i < ga; ++i) {
+          const double x = v1[i], d = d1[i];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const double y = row[(c * 3 + 0) * G + g1 + i];
-          X[c] = fma(y, x, X[c]);
-          J[c][0] = fma(y, d, J[c][0]);
-          J[c][1] = fma(row[(c * 3 + 1) * G + g1 + i], x, J[c][1]);
-          J[c][2] = fma(row[(c * 3 + 2) * G + g1 + i], x, J[c][2]);
+          for (int c = 0; c < 3; ++c) {
+            const double y = row[(c * 3 + 0) * G + g1 + i];
+            X[c] = fma(y, x, X[c]);
+            J[c][0] = fma(y, d, J[c][0]);
+            J[c][1] = fma(row[(c * 3 + 1) * G + g1 + i], x, J[c][1]);
+            J[c][2] = fma(row[(c * 3 + 2) * G + g1 + i], x, J[c][2]);
+          }
         }
+      } else {
+        const int at[3] = {q1, q2, q3};
+        geo_eval<3>(v, at, X, J);
       }
       const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) +
                          J[0][1] * (J[1][2] * J[2][0] - J[1][0] * J[2][2]) +
@@ -523,21 +538,22 @@ __global__ void __launch_bounds__(kLoad * RG) load_kernel(PV v, int c2, int c3, 
 }
 
 // RG groups of rows at once; a net too fine for their shared memory takes one
-// (a block's rows reach over at most all its control points of direction 1).
-template <int P, int RG = (P <= 3 ? 4 : 2)>
+// (a block's rows reach over at most all its control points of direction 1),
+// and one too fine for that the map point by point.
+template <int P, int RG = (P <= 3 ? 4 : 2), bool ROWS = true>
 igafd_status load_p(const PV &v, const double *fq, double *b, cudaStream_t s) {
   constexpr int A = P + 1, TE = kLoad / A;
-  const size_t smem = sizeof(double) * std::max((size_t)9 * v.gm[0] * RG, (size_t)A * A * kLoad);
-  if constexpr (RG > 1)
-    if (smem > kMaxSmem) return load_p<P, 1>(v, fq, b, s);
+  const size_t smem = sizeof(double) * std::max(ROWS ? (size_t)9 * v.gm[0] * RG : 0, (size_t)A * A * kLoad);
+  if constexpr (ROWS)
+    if (smem > kMaxSmem) return load_p<P, 1, (RG > 1)>(v, fq, b, s);
   static std::atomic<unsigned long long> smem_set{0};
-  IGAFD_TRY(allow_smem(load_kernel<P, RG>, smem_set));
+  IGAFD_TRY(allow_smem(load_kernel<P, RG, ROWS>, smem_set));
   const int tiles = (v.nel[0] + TE - 1) / TE;
   for (int c3 = 0; c3 < std::min(A, v.nel[2]); ++c3)
     for (int c2 = 0; c2 < std::min(A, v.nel[1]); ++c2)
       for (int par = 0; par < std::min(2, tiles); ++par) {
         const int ne2 = (v.nel[1] - c2 + A - 1) / A, ne3 = (v.nel[2] - c3 + A - 1) / A;
-        load_kernel<P, RG><<<dim3(ne2 * ne3, (tiles - par + 1) / 2), kLoad * RG, smem, s>>>(v, c2, c3, ne2, par, fq, b);
+        load_kernel<P, RG, ROWS><<<dim3(ne2 * ne3, (tiles - par + 1) / 2), kLoad * RG, smem, s>>>(v, c2, c3, ne2, par, fq, b);
         IGAFD_LAUNCHED(1);
         IGAFD_CUDA(cudaGetLastError());
       }
@@ -635,9 +651,12 @@ struct Runner {
     a.ld = P->stencil_half ? P->sh_ld : P->Np;
     a.H = P->stencil_half ? P->sh_H : 0;
     const int km = P->kctrl ? P->dir[0].km : 0;
-    const size_t smem0 = (size_t)(9 * P->dir[0].gm + km) * sizeof(double);
+    size_t smem0 = (size_t)(9 * P->dir[0].gm + km) * sizeof(double);
+    const bool rows = smem0 <= kMaxSmem;
+    if (!rows) smem0 = 0;
     static std::atomic<unsigned long long> smem_set{0};
-    IGAFD_TRY(allow_smem(points_kernel, smem_set));
+    IGAFD_TRY(allow_smem(points_kernel<true>, smem_set));
+    const auto points = rows ? points_kernel<true> : points_kernel<false>;
     size_t smem1 = 0;                       // rows' points of a dir1 block
     for (int i = 0; i < P->n[0]; i += kRows) {
       int lo, hi;
@@ -662,7 +681,7 @@ struct Runner {
         elements(2, i3, i3 + a.c3, &lo, &hi);
         have = std::max(have, lo);
         if (hi > have) {
-          points_kernel<<<dim3(a.C2, (hi - have) * nq), kThr, smem0, s>>>(a, have);
+          points<<<dim3(a.C2, (hi - have) * nq), kThr, smem0, s>>>(a, have);
           IGAFD_LAUNCHED(1);
           have = hi;
         }
