@@ -413,8 +413,10 @@ igafd_status igafd_setup_prec(igafd_patch *patch, void *stream);
  * iterative refinement of the eigenvectors (Ogita and Aishima, 2018) and
  * exact rotations of nearly degenerate pairs, accepted only if
  * max |U~^T U~ - I| <= 1e-12 and the off-diagonal of U~^T K~ U~ is <= 1e-12
- * of its diagonal; FP64 cyclic Jacobi otherwise; 1 = FP64 Jacobi for every direction. igafd_patch_info.eig_refined reports the
- * route each direction took. Other values: IGAFD_ERR_ARG. */
+ * of its diagonal; FP64 cyclic Jacobi otherwise, for n_k > 128 also where
+ * more than two eigenvalues lie within 1e-5 of the largest of the one below;
+ * 1 = FP64 Jacobi for every direction. igafd_patch_info.eig_refined reports
+ * the route each direction took. Other values: IGAFD_ERR_ARG. */
 igafd_status igafd_set_eig_route(igafd_patch *patch, int route);
 
 /* Polls after which a device wait of the FP64 FD on the tensor cores gives up

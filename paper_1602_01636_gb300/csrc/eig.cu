@@ -622,11 +622,20 @@ __global__ void __launch_bounds__(1024) tri32_kernel(EigJob *jobs, int allow_fas
 // once). Every pass over a matrix walks its rows, coalesced; L1 holds much of
 // it up to n of about 200. One CTA does the start up to T's eigenvectors;
 // back32_kernel takes them back to the pencil's, columns spread over CTAs.
-// Measured at p = 3 before the degree limit below (the work hardly depends on
-// p), the whole eigendecomposition with the refinement: 1.5 ms at n = 150,
-// 2.1 at 192, 6 at 300, 24 at 512, where FP64 Jacobi took 73, 161, 647 and 3600
+// Measured, set-up of P with p = 1 and 2 on uniform knots: 1.5 ms at n = 150,
+// 6.1 at 300, 25.6 at 513, where FP64 Jacobi takes 73-80, 640-690 and 3200-3600
 // ms. Bound by the tridiagonalisation's passes over the matrix (one CTA).
 constexpr int kBigMaxN = 1024;
+
+// Spectra with more than kBigClose eigenvalues within kInvCluster ||T|| of the
+// one below, which the start cannot tell apart, go to the FP64 Jacobi at once:
+// of 39 pencils with n = 150 to 900 on uniform, uneven, graded and repeated knots
+// and with span scalings, the 18 with three or more all failed the acceptance
+// test, 17 of the others met it (uniform knots up to n = 640). Graded knots have
+// hundreds of them, in runs that one thread would orthogonalise: with spans
+// graded by 10^3 the set-up took 870 ms at n = 300 and 6.4 s at 513, now 555 ms
+// and 3.2 s, Jacobi alone 550 ms and 3.2 s.
+constexpr int kBigClose = 2;
 
 // Degrees up to which the route takes n > kFastMaxN. From p = 3 on, pencils on
 // uniform knots have pairs of outlier eigenvalues (one function at either end)
@@ -860,7 +869,10 @@ __global__ void __launch_bounds__(1024) big32_kernel(EigJob *jobs, int allow_fas
   // (eigenvalues closer than kInvCluster ||T||) are solved in turn by its first
   // member's thread and orthogonalised against each other
   if (tid < n) s_start[tid] = (tid == 0 || lam[tid] - lam[tid - 1] > kInvCluster * tn) ? 1 : 0;
-  __syncthreads();
+  if (__syncthreads_count(tid < n && !s_start[tid]) > kBigClose) {
+    if (tid == 0) *jb.state = 1;
+    return;
+  }
   const float floor = 1.2e-7f * tn;
   if (tid < n && s_start[tid]) {
     int last = tid;
