@@ -22,18 +22,22 @@
 // FP64 once. A product's error is relative to the largest entries of its row
 // and column: in units of 2^-53 of their norms 0.1-0.2 for rows along an
 // eigenvector of degree 1 (an FP64 chain: 6-9), 18 for one large entry among
-// 127 equal ones that are smaller by any factor (chain: 47). The divide by D_1 (+) D_2 (+) D_3
-// multiplies the integer result before that rounding. No FP64 instruction is
-// executed (each would issue at the 2-per-clock rate).
+// 127 equal ones that are smaller by any factor (chain: 47). The divide by
+// D_1 (+) D_2 (+) D_3 multiplies the integer result before that rounding. The
+// digits' path executes no FP64 instruction (each would issue at the
+// 2-per-clock rate).
 //
 // Measured: 212 us per apply at n = 128 (SIMT: 3.10 ms), 110 us at (95, 61, 77)
-// (SIMT: 0.98 ms). A pass at n = 128 takes the phases of its one tile per SM in
-// turn: reading and splitting the rows (6 us), the MMAs with the summation of
-// their accumulators (the MMAs alone 5 us), the last rounding (2.5 us), and
-// about 6 us between two launches. With groups 1 to 3 in fewer, larger sums
-// (eight instead of fifteen steps at K = 128) an apply took 172 and 94 us, but
-// rows whose digits add up with one sign passed 2^24 and lost up to 3000 units
-// of 2^-53.
+// (SIMT: 0.98 ms), 1.41 ms at n = 192 (SIMT: 13.8 ms). A pass at n = 128 takes the
+// phases of its one tile per SM in turn, nothing beside them: reading and
+// splitting the rows (6 us), the MMAs with the summation of their accumulators
+// (the MMAs alone 5 us), the last rounding (2.5 us), and about 6 us between two
+// launches. A profile shows 23 % of the issue slots and 10 % of the tensor pipe
+// in use; waiting for instructions is the largest stall (the unrolled steps
+// miss the instruction cache), but the steps of a group as a loop took as long.
+// With groups 1 to 3 in fewer, larger sums (eight instead of fifteen steps at
+// K = 128) an apply took 172 and 94 us, but rows whose digits add up with one
+// sign passed 2^24 and lost up to 3000 units of 2^-53.
 //
 // A CTA takes 128 rows (the other directions' indices) and up to 128 columns.
 // A's digits live in tensor memory (6 slices of K/2 columns: 384 of 512 at

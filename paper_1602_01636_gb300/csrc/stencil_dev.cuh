@@ -2,16 +2,16 @@
 // the stencil layout, the arguments, the per-CTA pipeline and the ring set-up.
 #pragma once
 // y = A x with A stored as a (2p+1)^d-point FP64 stencil, offset-major:
-// S[o][row] with row stride Np (N rounded up to the tile), o = sum_k
+// S[o][row] with row stride Np (N rounded up to kTile), o = sum_k
 // (delta_k + p)(2p+1)^(k-1) (Section 2.1: an interior row of A couples to
 // (2p+1)^d columns). Also r = b - A x (true residual).
 //
 // On GB300 the 343 FP64 FMAs of a p = 3 row take longer on the FP64 pipe
 // (2 FMA/clk/SM) than its 2.7 KB of coefficients take to stream from HBM, so
 // the kernel is built to keep the FP64 pipe fed from shared memory: a
-// persistent grid of CTAs walks 256-row tiles; for every (delta_2, delta_3)
-// group a producer warp brings the 2p+1 coefficient runs of the tile
-// (contiguous 2 KB each) and the contiguous window of x they multiply into a
+// persistent grid of CTAs walks tiles of 64 to 256 rows (tile_rows); for every
+// (delta_2, delta_3) group a producer warp brings the 2p+1 coefficient runs of
+// the tile (contiguous) and the contiguous window of x they multiply into a
 // shared-memory ring with bulk asynchronous copies (cp.async.bulk, completion
 // on mbarriers), several groups ahead of the eight compute warps. x is read
 // from a copy with a zero halo of p planes on both ends, and couplings that
@@ -158,8 +158,9 @@ struct Geom {
 // offset o below the centre (delta < 0) is the mirrored offset's run shifted
 // by off(delta) rows, S[mirror(o) - oc][shH + row0 + off ...], fetched from
 // the even row at or before its start so that every bulk copy is 16-byte
-// aligned; every run is RS = kTile + 2 rows long and the compute warps read a
-// mirrored run one row later when its start was odd.
+// aligned; every run is two rows longer than the tile (RS = kTile + 2 apart in
+// shared memory) and the compute warps read a mirrored run one row later when
+// its start was odd.
 template <int DIM, int P, int MODE, int kStages, int R, bool HALF = false>
 __device__ __forceinline__ void stencil_cta(const StencilArgs &a, long long vb, long long vgrid,
                                             double *ring, uint64_t *full, uint64_t *empty,
