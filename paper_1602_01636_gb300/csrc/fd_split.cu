@@ -733,6 +733,7 @@ size_t pass_smem(int Kp) {
 }  // namespace
 
 struct FDSplit {
+  unsigned char *mem;         // one allocation for all below
   unsigned char *img[3][2];   // [direction][0: U_k^T, 1: U_k]
   int *eb[3][2];
   int *col[3];                // column scalings of U_k (exponents), then its rows' range (2)
@@ -752,31 +753,44 @@ igafd_status igafd_fd_split_init(igafd_patch *P, cudaStream_t s) {
     P->split = (FDSplit *)calloc(1, sizeof(FDSplit));
     if (!P->split) return IGAFD_ERR_OOM;
   }
-  ImgBatch b[2] = {};
-  int rows = 0;
-  for (int k = 0; k < P->dim; ++k) {
-    const int n = P->n[k];
-    if (!P->split->col[k] && cudaMalloc(&P->split->col[k], (n + 2) * sizeof(int)) != cudaSuccess) {
-      cudaGetLastError();
-      return IGAFD_ERR_OOM;
-    }
-    for (int d = 0; d < 2; ++d) {
-      ImgJob &J = b[d].j[k];
-      J.U = P->U[k]; J.n = n; J.Np = pad(n, 16); J.Kp = pad(n, 32);
-      J.transpose = d == 0;
-      const size_t sz = (size_t)kSlices * ((J.Kp + 63) / 64) * J.Np * 128;
-      if ((!P->split->img[k][d] && cudaMalloc(&P->split->img[k][d], sz) != cudaSuccess) ||
-          (!P->split->eb[k][d] && cudaMalloc(&P->split->eb[k][d], J.Np * sizeof(int)) != cudaSuccess)) {
+  FDSplit &S = *P->split;
+  if (!S.mem) {
+    // sizes first, then addresses, each on a 256-byte boundary
+    for (int set = 0; set < 2; ++set) {
+      size_t at = 0;
+      auto take = [&](size_t bytes) {
+        unsigned char *q = S.mem + (set ? at : 0);
+        at += (bytes + 255) / 256 * 256;
+        return q;
+      };
+      for (int k = 0; k < P->dim; ++k) {
+        const int n = P->n[k], Np = pad(n, 16), Kp = pad(n, 32);
+        S.col[k] = (int *)take((n + 2) * sizeof(int));
+        for (int d = 0; d < 2; ++d) {
+          S.img[k][d] = take((size_t)kSlices * ((Kp + 63) / 64) * Np * 128);
+          S.eb[k][d] = (int *)take(Np * sizeof(int));
+        }
+      }
+      if (!set && cudaMalloc(&S.mem, at) != cudaSuccess) {
         cudaGetLastError();
+        S.mem = nullptr;
         return IGAFD_ERR_OOM;
       }
-      J.img = P->split->img[k][d];
-      J.eb = P->split->eb[k][d];
-      J.col = P->split->col[k];
-      J.range = J.col + n;
-      rows = J.Np > rows ? J.Np : rows;
     }
   }
+  ImgBatch b[2] = {};
+  int rows = 0;
+  for (int k = 0; k < P->dim; ++k)
+    for (int d = 0; d < 2; ++d) {
+      ImgJob &J = b[d].j[k];
+      J.U = P->U[k]; J.n = P->n[k]; J.Np = pad(J.n, 16); J.Kp = pad(J.n, 32);
+      J.transpose = d == 0;
+      J.img = S.img[k][d];
+      J.eb = S.eb[k][d];
+      J.col = S.col[k];
+      J.range = J.col + J.n;
+      rows = J.Np > rows ? J.Np : rows;
+    }
   for (int d = 0; d < 2; ++d) split_image_kernel<<<dim3(rows, P->dim), 256, 0, s>>>(b[d]);
   IGAFD_LAUNCHED(2);
   IGAFD_CUDA(cudaGetLastError());
@@ -785,13 +799,7 @@ igafd_status igafd_fd_split_init(igafd_patch *P, cudaStream_t s) {
 
 void igafd_fd_split_free(igafd_patch *P) {
   if (!P || !P->split) return;
-  for (int k = 0; k < 3; ++k) {
-    for (int d = 0; d < 2; ++d) {
-      cudaFree(P->split->img[k][d]);
-      cudaFree(P->split->eb[k][d]);
-    }
-    cudaFree(P->split->col[k]);
-  }
+  cudaFree(P->split->mem);
   free(P->split);
   P->split = nullptr;
 }
