@@ -28,6 +28,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 namespace {
@@ -171,12 +172,19 @@ __global__ void __launch_bounds__(kThreads) tc_pass_kernel(PassArgs a) {
   // per-tile power-of-two scale for FP16 operands
   float a_scale = 1.0f;
   if (OP == OP_FP16) {
+    // (the type is decided outside the loop, so that its loads can overlap)
     float mx = 0.0f;
-    for (int i = tid; i < mrows * K; i += kThreads) {
-      const long long idx = (m0 + i / K) * K + i % K;
-      const float v = a.in_f64 ? f64_to_f32(((const double *)a.in)[idx]) : ((const float *)a.in)[idx];
-      mx = fmaxf(mx, fabsf(v));
-    }
+    auto scan = [&](auto *in) {
+#pragma unroll 4
+      for (int i = tid; i < mrows * K; i += kThreads) {
+        float v;
+        if constexpr (sizeof(*in) == 8) v = f64_to_f32(in[i]);
+        else v = in[i];
+        mx = fmaxf(mx, fabsf(v));
+      }
+    };
+    if (a.in_f64) scan((const double *)a.in + m0 * K);
+    else scan((const float *)a.in + m0 * K);
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0) s_red[warp] = mx;
     __syncthreads();
@@ -254,30 +262,38 @@ __global__ void __launch_bounds__(kThreads) tc_pass_kernel(PassArgs a) {
             : "memory");
     }
     // stage A: warp w takes rows 16w..16w+15, lane l columns k0+2l, k0+2l+1;
-    // all sixteen loads are issued before the swizzled, rounded stores
+    // all sixteen loads are issued before the swizzled, rounded stores (and
+    // before FP64 input is converted: converted as it came, each load waited
+    // for the one before it)
     {
       float2 v[16];
       const bool vec = a.in_aligned && (K % 2 == 0) && (k0 + kKC <= K);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int rr = warp * 16 + i;
+      auto load = [&](auto *in, auto *d) {               // d: pairs of in's type
+        using D = std::remove_reference_t<decltype(*d)>;
         const int k = k0 + 2 * lane;
-        v[i] = make_float2(0.f, 0.f);
-        if (rr < mrows) {
-          const long long idx = (m0 + rr) * K + k;
-          if (vec) {
-            if (a.in_f64) {
-              const double2 d = *reinterpret_cast<const double2 *>((const double *)a.in + idx);
-              v[i] = make_float2(f64_to_f32(d.x), f64_to_f32(d.y));
-            } else {
-              v[i] = *reinterpret_cast<const float2 *>((const float *)a.in + idx);
-            }
-          } else {
-            if (k < K) v[i].x = a.in_f64 ? f64_to_f32(((const double *)a.in)[idx]) : ((const float *)a.in)[idx];
-            if (k + 1 < K)
-              v[i].y = a.in_f64 ? f64_to_f32(((const double *)a.in)[idx + 1]) : ((const float *)a.in)[idx + 1];
+        in += (m0 + warp * 16) * K + k;
+        if (vec) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            d[i] = D{};
+            if (warp * 16 + i < mrows) d[i] = *reinterpret_cast<const D *>(in + (long long)i * K);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            d[i] = D{};
+            if (warp * 16 + i < mrows && k < K) d[i].x = in[(long long)i * K];
+            if (warp * 16 + i < mrows && k + 1 < K) d[i].y = in[(long long)i * K + 1];
           }
         }
+      };
+      if (a.in_f64) {
+        double2 d[16];
+        load((const double *)a.in, d);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = make_float2(f64_to_f32(d[i].x), f64_to_f32(d[i].y));
+      } else {
+        load((const float *)a.in, v);
       }
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
