@@ -46,7 +46,7 @@ igafd_status launch_one(StencilArgs &a, int num_sms, cudaStream_t s, long long *
   static std::atomic<int> per_sm_tab[64];
   int per_sm = 1;
   IGAFD_TRY(per_sm_of(kern, kBlock, smem, attr_set, per_sm_tab, &per_sm));
-  a.tile = tile_rows(a.N, num_sms, per_sm, 32 * R);
+  a.tile = tile_rows(a.N, num_sms, per_sm, 32 * R, a.partial ? kSolveTile : 64);
   a.ntiles = (a.N + a.tile - 1) / a.tile;
   long long grid = (long long)num_sms * per_sm;
   if (grid > a.ntiles) grid = a.ntiles;

@@ -28,6 +28,7 @@
 namespace {
 
 constexpr int kTile = 256;                        // rows per tile at most (StencilArgs::tile in use)
+constexpr int kSolveTile = 128;                   // and at least in a solve (tile_rows)
 // ring depths (offset groups in flight per CTA) the kernel is built for; the
 // autotuner picks one per (dimension, degree, sizes), default kStagesDefault
 constexpr int kStagesDefault = 4;
@@ -474,10 +475,16 @@ igafd_status per_sm_of(Kern kern, int block, size_t smem, std::atomic<unsigned l
 // tiles only, the last round of a mid-sized patch ran on few CTAs and a small
 // patch on few SMs: (61, 90, 47) at p = 4 took 373 us, now 319 (299 us of FP64
 // work); (20, 20, 20) at p = 3 took 35 us, now 24. Ties go to the larger tile.
-inline int tile_rows(long long N, int sms, int per_sm, int step) {
+// The products of a solve take tiles of kSolveTile rows or more: a batch runs the
+// same tiles (its results are the single solves' bit for bit) for many problems
+// at once, where the SMs are never idle and small tiles only cost (12 problems
+// of 16 to 48 functions per direction, one group each, BF16: 6.34 ms with tiles
+// down to 64 rows, 5.95 with 128, 5.77 with 256 only; the same problems one by
+// one 13.4, 13.6 and 14.1 ms).
+inline int tile_rows(long long N, int sms, int per_sm, int step, int lowest) {
   int best = kTile;
   double cost = -1.0;
-  for (int h = kTile; h >= 64; h -= step) {
+  for (int h = kTile; h >= lowest; h -= step) {
     const long long tiles = (N + h - 1) / h, ctas = (long long)sms * per_sm;
     const long long rounds = (tiles + ctas - 1) / ctas;
     const double rows = (double)h * (rounds > 1 ? per_sm : (double)((tiles + sms - 1) / sms));
